@@ -93,6 +93,7 @@ inline void fixed_coef(const lbm13_params &p, const double *D, const lbm13_bound
     x.Fx0 = (1.0 - k.rho_ref) * k.gx;
     x.Fy0 = (1.0 - k.rho_ref) * k.gy;
     x.q = b.heat;
+    x.source = b.heat != 0.0;
     x.top = fx_mag(std::max({std::fabs(x.Fx0), std::fabs(x.Fy0), std::fabs(x.q)}));
     // with that, |F| is below 1.2 and |j + F/2| below 10.6 of the node's unit
     ok = ok && std::fabs(k.gx) < 1.0 / 64 && std::fabs(k.gy) < 1.0 / 64;
@@ -121,7 +122,10 @@ inline void fixed_coef(const lbm13_params &p, const double *D, const lbm13_bound
         double f[Q] = {};
         f[j] = 1e-9;
         collide_plain<false>(f, k);
-        for (int i = 0; i < Q; ++i) row[i] += std::fabs(f[i]) * real(1e9);
+        // the rest population may be 2^kFixRest times as large as the others, and
+        // what it keeps of itself is not in the integers
+        for (int i = 0; i < Q; ++i)
+            row[i] += j > 0 ? std::fabs(f[i]) * real(1e9) : i > 0 ? std::fabs(f[i]) * real(1e9) * (1 << kFixRest) : 0;
     }
     // momentum flux at |j| < 10.6 / 32, rho > 0.59; the work of F and the source
     const real flux = lXX * real(10.6 * 10.6 / 0.59 / 32), p1 = product(r1) + real(0.6) * A1 + real(0.1),
@@ -129,7 +133,17 @@ inline void fixed_coef(const lbm13_params &p, const double *D, const lbm13_bound
                s1 = std::fabs(s[1]);
     const real extra[4] = {28 * dE + s0, 15 * dE + s1 + p1 + flux, 2 * dE + s0 / 2 + 2 * s1 + p1 + 2 * p9 + 17 * flux,
                            24 * dE + s0 / 4 + s1 / 2 + p9 + 4 * flux};
-    for (int j = 0; j < Q; ++j) ok = ok && row[j] + extra[j == 0 ? 0 : j < 5 ? 1 : j < 9 ? 2 : 3] < real(15.9);
+    for (int j = 1; j < Q; ++j) ok = ok && row[j] + extra[j < 5 ? 1 : j < 9 ? 2 : 3] < real(15.9);
+    // the scalar block's increment of the rest population, and what shells 9 and 5
+    // are rounded from; with t > 0 the force's part is below 4 units too
+    real in0 = 4 + s0, in9 = 0, in5 = 0;
+    for (int l = 0; l < 4; ++l) {
+        const real w = l == 0 ? 1 << kFixRest : 4;
+        in0 += w * std::fabs(B[0][l]);
+        in9 += w * std::fabs(B[0][l] + 2 * B[1][l]);
+        in5 += w * std::fabs(B[0][l] + 3 * B[1][l]);
+    }
+    ok = ok && in0 < real(15.9) && in9 < real(15.9) && in5 < real(15.9);
     x.on = ok ? 1 : 0;
 }
 

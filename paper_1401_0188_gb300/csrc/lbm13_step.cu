@@ -47,8 +47,9 @@ namespace {
 // register caps keep 6 blocks (24 warps) per SM for FP32 and 5 for the forced
 // two-row FP32 variant, without spills: more warps keep more population loads in
 // flight.  FP64 (the collision in integers) takes 7 blocks at 72 registers although
-// a few words spill: its warps wait for their chains of integer instructions, and
-// 2048^2 measured 201 / 188 / 181 / 184 / 195 us a step with 5 / 6 / 7 / 8 / 9 blocks.
+// 26 words spill (73 with a force): its warps wait for their chains of integer
+// instructions; 2048^2 measured 254 / 254 / 263 us a step with 5 / 6 / 7 blocks while
+// the collision held more values, and 213 / 211 with 6 / 7 (279 / 276 with a force) now.
 template <typename T, typename C, bool Force, int R>
 __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 7 : Force && R == 2 ? 5 : 6) step_kernel(const StepArgs<T, C> a)
 {
