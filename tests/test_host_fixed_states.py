@@ -2,7 +2,8 @@
 states that flows hold: density, temperature and velocity deviations of very
 different sizes, where the rest population is 30 times the diagonals or a thousandth
 of the unit links.  Its error against 113 bits is no larger than that of the FP64
-collision, and nodes at the ends of its range stay inside 63 bits."""
+collision, mirrored nodes collide to mirrored populations bit for bit, and nodes at
+the ends of its range stay inside 63 bits."""
 import numpy as np
 import pytest
 
@@ -13,6 +14,9 @@ from paper_1401_0188_gb300 import workloads as W
 
 lib = H.lib  # the compiled harness (a module fixture)
 Q = 13
+# what mirroring x, mirroring y and turning by half a turn make of the links
+MIRRORS = {"x": [0, 3, 2, 1, 4, 6, 5, 8, 7, 11, 10, 9, 12], "y": [0, 1, 4, 3, 2, 8, 7, 6, 5, 9, 12, 11, 10],
+           "xy": [0, 3, 4, 1, 2, 7, 8, 5, 6, 11, 12, 9, 10]}
 # amplitudes of density, velocity and temperature
 SIZES = {"mixed": (2e-3, 1e-2, 2e-3), "density": (1e-2, 1e-4, 0.0), "temperature": (0.0, 1e-4, 5e-3),
          "slow": (1e-2, 1e-6, 5e-3), "fast": (1e-5, 1e-2, 1e-5), "flow": (1e-4, 1e-2, 1e-4), "faint": (1e-6, 1e-6, 1e-6)}
@@ -49,6 +53,27 @@ def test_integer_collision_is_no_less_exact_than_fp64_at_flow_states(lib, params
     # of each population: 4000 nodes estimate an rms to 1.1%; those whose error in
     # FP64 is little more than the last rounding have at most a quarter more
     assert (rms(ei) <= 1.25 * rms(ep)).all(), rms(ei) / rms(ep)
+
+
+@pytest.mark.parametrize("mirror", list(MIRRORS))
+@pytest.mark.parametrize("bound", list(H.BOUNDS))
+def test_mirrored_nodes_collide_to_mirrored_populations(lib, bound, mirror):
+    b = H.BOUNDS[bound]
+    m = MIRRORS[mirror]
+    image = dict(b, gx=b["gx"] * (-1 if "x" in mirror else 1), gy=b["gy"] * (-1 if "y" in mirror else 1))
+    rng = np.random.default_rng(2)
+    p = H.PARAMS["pstar"]()
+    f = np.concatenate([_states(p, s, 2000, rng, 1e-3) for s in SIZES.values()] + [H._states("even", 2000, rng)])
+    # few significant bits: sums that end in halves are common
+    g = f.copy()
+    g[::2] = np.float32(g[::2])
+    g[1::4] = np.round(g[1::4] * 2.0 ** 20) * 2.0 ** -20
+    for x in (f, g):
+        a = H._run(lib, p, b, x)
+        c = H._run(lib, p, image, x[:, m])
+        assert np.array_equal(a[1], c[1])
+        assert np.array_equal(a[2][2][:, m], c[2][2])   # the whole collision
+        assert np.array_equal(a[2][1][:, m], c[2][1])   # the FP64 one it replaces
 
 
 @pytest.mark.parametrize("bound", list(H.BOUNDS))
