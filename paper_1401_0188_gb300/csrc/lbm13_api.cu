@@ -241,12 +241,14 @@ ReadArgs<T> read_args(lbm13_t h)
     a.pitch = h->pitch;
     a.plane = h->plane;
     a.rest.E0 = h->p.E0;
+    a.rest.T0 = (h->p.E0 + 28.0) / 26.0;
     a.rest.eps0 = h->derived[6] + h->p.c_epsE * h->p.E0;
     a.rest.vpi0 = h->p.c_vpi_rho + h->p.c_vpi_E * h->p.E0;
     a.gx = h->b.gx;
     a.gy = h->b.gy;
     a.rho_ref = h->b.rho_ref;
     a.heat = h->b.heat;
+    a.force = h->b.gx != 0.0 || h->b.gy != 0.0;
     a.fx = h->fr;
     return a;
 }

@@ -46,49 +46,61 @@ __global__ void init_kernel(T *f, int nx, int ny, long long pitch, long long pla
 
 // -------------------------------------------------------------- moments
 
-// The read-out of one node in FP64 (nodes that the integer one does not take):
-// bits 0 .. 12 the absolute moments, then u_x, u_y, T, p and the Sec. 7 energy.
+// The selected fields of one node in FP64, in order: bits 0 .. 12 the absolute
+// moments, then u_x, u_y, T, p and the Sec. 7 energy.  All: moments other than rho, E
+// and the momentum may be among them (their 25 operations are left out otherwise).
+constexpr unsigned kOtherMoments = 0x1fccu;
+template <bool All, typename T, typename Put>
+__device__ __forceinline__ void put_fields(const ReadArgs<T> &a, const double (&f)[Q], unsigned mask, Put put)
+{
+    Mom<double> d;
+    forward(f, d);
+    if (mask & 0x1u) put(1.0 + d.rho);
+    if (mask & 0x2u) put(a.rest.E0 + d.E);
+    if (All && (mask & 0x4u)) put(a.rest.eps0 + d.eps);
+    if (All && (mask & 0x8u)) put(a.rest.vpi0 + d.vpi);
+    if (mask & 0x10u) put(d.jx);
+    if (mask & 0x20u) put(d.jy);
+    if (All && (mask & 0x40u)) put(d.qx);
+    if (All && (mask & 0x80u)) put(d.qy);
+    if (All && (mask & 0x100u)) put(d.rx);
+    if (All && (mask & 0x200u)) put(d.ry);
+    if (All && (mask & 0x400u)) put(d.XX);
+    if (All && (mask & 0x800u)) put(d.XY);
+    if (All && (mask & 0x1000u)) put(d.XXe);
+    if (!(mask >> 13)) return;
+    const double T0 = a.rest.T0;
+    double ux, uy, dT, dp;
+    macro_dev(a, d.rho, d.E, d.jx, d.jy, ux, uy, dT, dp);
+    if (mask & 0x2000u) put(ux);
+    if (mask & 0x4000u) put(uy);
+    if (mask & 0x8000u) put(T0 + dT);
+    if (mask & 0x10000u) put(T0 + dp);
+    if (mask & 0x20000u) put(a.rest.E0 + d.E - 6.5 * (ux * ux + uy * uy));
+}
 template <typename T>
-__device__ __noinline__ double node_field(const ReadArgs<T> &a, const T (&raw)[Q], int b)
+__device__ __noinline__ void put_fields_plain(const ReadArgs<T> &a, const T (&raw)[Q], unsigned mask, double *o, long long n)
 {
     double f[Q];
     widen(raw, f);
-    Mom<double> d;
-    forward(f, d);
-    const double m[Q] = {1.0 + d.rho, a.rest.E0 + d.E, a.rest.eps0 + d.eps, a.rest.vpi0 + d.vpi, d.jx, d.jy, d.qx,
-                         d.qy, d.rx, d.ry, d.XX, d.XY, d.XXe};
-    if (b < Q) return m[b];
-    const double rho = m[0], w = rho - a.rho_ref;
-    const double ux = (d.jx - 0.5 * w * a.gx) / rho, uy = (d.jy - 0.5 * w * a.gy) / rho;
-    const double p = (m[1] + 28.0 * rho) / 26.0 - (d.jx * d.jx + d.jy * d.jy) / (2.0 * rho) - 0.5 * a.heat;
-    return b == 13 ? ux : b == 14 ? uy : b == 15 ? p / rho : b == 16 ? p : m[1] - 6.5 * (ux * ux + uy * uy);
-}
-
-// The selected fields of one node per thread.  The integer read-out leaves one
-// conversion and at most a few FP64 operations per selected field (8192^2 FP32,
-// rho, u and T: see the header of lbm13_fixed_io.cuh).
-template <typename T>
-__global__ void __launch_bounds__(128) moments_kernel(const ReadArgs<T> a, double *__restrict__ out, unsigned mask)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= a.nx) return;
-    T f[Q];
-    load_node(a, (long long)y * a.pitch + x, f);
-    const long long n = (long long)a.nx * a.ny;
-    double *o = out + (long long)y * a.nx + x;
-    const auto put = [&](double v) {
+    put_fields<true>(a, f, mask, [&](double v) {
         *o = v;
         o += n;
-    };
+    });
+}
+
+// The same for FP32 storage in integers.
+template <typename Put>
+__device__ __forceinline__ void put_fields_fixed(const ReadArgs<float> &a, const float (&f)[Q], unsigned mask, Put put,
+                                                 double *o, long long n)
+{
     FxSums s;
     FxMacro m;
     if (!fx_sums(f, s) || ((mask >> 13) != 0u && !fx_macro(s, a.fx, m))) {
-        T g[Q];  // f itself stays in registers
+        float g[Q];  // f itself stays in registers
 #pragma unroll
         for (int j = 0; j < Q; ++j) g[j] = f[j];
-        for (int b = 0; b < 18; ++b)
-            if ((mask >> b) & 1u) put(node_field(a, g, b));
+        put_fields_plain(a, g, mask, o, n);
         return;
     }
     if (mask & 0x1u) put(1.0 + s.value(s.rho()));
@@ -109,12 +121,39 @@ __global__ void __launch_bounds__(128) moments_kernel(const ReadArgs<T> a, doubl
     if (mask & 0x1000u) put(s.value(s.X9 - 4 * s.X1));
     if (mask & 0x2000u) put(s.value(m.ux));
     if (mask & 0x4000u) put(s.value(m.uy));
-    const double T0 = (a.rest.E0 + 28.0) / 26.0;
+    const double T0 = a.rest.T0;
     if (mask & 0x8000u) put(T0 + s.value(m.dT));
     if (mask & 0x10000u) put(T0 + s.value(m.dp));
     if (mask & 0x20000u) {
         const double ux = s.value(m.ux), uy = s.value(m.uy);
         put(a.rest.E0 + s.energy() - 6.5 * (ux * ux + uy * uy));
+    }
+}
+
+// The selected fields of one node per thread.  The integer read-out of FP32 storage
+// leaves one conversion and at most a few FP64 operations per selected field (8192^2
+// FP32, rho, u and T: see the header of lbm13_fixed_io.cuh).
+template <typename T>
+__global__ void __launch_bounds__(128) moments_kernel(const ReadArgs<T> a, double *__restrict__ out, unsigned mask)
+{
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y;
+    if (x >= a.nx) return;
+    T f[Q];
+    load_node(a, (long long)y * a.pitch + x, f);
+    const long long n = (long long)a.nx * a.ny;
+    double *o = out + (long long)y * a.nx + x;
+    const auto put = [&](double v) {
+        *o = v;
+        o += n;
+    };
+    if constexpr (sizeof(T) == 8) {
+        if (mask & kOtherMoments)
+            put_fields<true>(a, f, mask, put);
+        else
+            put_fields<false>(a, f, mask, put);
+    } else {
+        put_fields_fixed(a, f, mask, put, o, n);
     }
 }
 
@@ -230,7 +269,7 @@ __device__ __forceinline__ void fields_pass(const ReadArgs<T> &a, const ReduceBu
 {
     __shared__ double res[kSums + kMax];
     const long long n = (long long)a.nx * a.ny;
-    const double T0 = (a.rest.E0 + 28.0) / 26.0;
+    const double T0 = a.rest.T0;
     double s[kSums] = {0, 0, 0, 0, 0, 0, 0, 0};
     unsigned long long mx[kMax] = {0, 0};
     for (long long i = (long long)block * kReduceThreads + threadIdx.x; i < n; i += (long long)b.nblocks * kReduceThreads) {

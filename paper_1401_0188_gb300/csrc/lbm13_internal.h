@@ -115,9 +115,9 @@ int linear_growth(const lbm13_params &p, const double *D, double ux, double uy, 
 int linear_growth_batch(const lbm13_params *p, const double *D, const double *ux, const double *uy, int count, int n,
                         double *growth, cudaStream_t s);
 
-// Rest moments used by the read-outs (double precision).
+// Rest moments and temperature used by the read-outs (double precision).
 struct Rest {
-    double E0, eps0, vpi0;
+    double E0, eps0, vpi0, T0;
 };
 
 // Arguments of the read-out and reduction kernels (always double).
@@ -129,6 +129,7 @@ struct ReadArgs {
     Rest rest;
     double gx, gy, rho_ref;
     double heat;  // energy source q: T is read half-way, (p* - q/2)/rho
+    int force;    // nonzero when g != 0
     ReadFix fx;   // the same in integers
 };
 

@@ -221,10 +221,12 @@ cudaError_t launch_totals(const StateView &v, int nblocks, double *scratch)
     a.pitch = v.pitch;
     a.plane = v.plane;
     a.rest.E0 = v.E0;
+    a.rest.T0 = (v.E0 + 28.0) / 26.0;
     a.gx = v.gx;
     a.gy = v.gy;
     a.rho_ref = v.rho_ref;
     a.heat = v.heat;
+    a.force = v.gx != 0.0 || v.gy != 0.0;
     a.fx = v.fx;
     return cudaLaunchKernelEx(&cfg, totals_kernel<T>, a, scratch);
 }

@@ -1,0 +1,145 @@
+"""Read-outs (csrc/lbm13_read.cuh) on the host, at the states that flows hold: a small velocity beside large deviations of
+density and temperature, and the other way round.  Against 113-bit arithmetic no
+reading is less exact than FP64 arithmetic with one rounding per
+operation gives it."""
+import ctypes as C
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+import test_host_fixed_states as S
+from paper_1401_0188_gb300 import lbm13, pstar
+from paper_1401_0188_gb300 import params as P
+from paper_1401_0188_gb300 import workloads as W
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1401_0188_gb300", "csrc")
+CUDA_INC = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+Q = 13
+
+SRC = r"""
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <cuda_runtime.h>
+#include "lbm13_coef.h"
+using std::isfinite;
+#include "lbm13_read.cuh"
+using namespace lbm13;
+#if __LDBL_MANT_DIG__ >= 113
+typedef long double quad;
+#else
+typedef __float128 quad;
+#endif
+
+// f [13][n]; out [n][8]: rho - 1, E - E0, j_x, j_y, u_x, u_y, T - T0, p - T0: the
+// kernels' node_dev (ei) and FP64 operation by operation (ep), errors
+template <typename T>
+static void read_all(const lbm13_params &p, const lbm13_boundary &b, int n, const T *f, double *value, double *ei, double *ep)
+{
+    ReadArgs<T> a{};
+    a.f = f;
+    a.nx = n;
+    a.ny = 1;
+    a.pitch = a.plane = n;
+    a.rest.E0 = p.E0;
+    a.rest.T0 = (p.E0 + 28.0) / 26.0;
+    a.gx = b.gx;
+    a.gy = b.gy;
+    a.rho_ref = b.rho_ref;
+    a.heat = b.heat;
+    a.force = b.gx != 0.0 || b.gy != 0.0;
+    read_fix(p.E0, b, a.fx);
+    for (int i = 0; i < n; ++i) {
+        double g[Q];
+        quad e[Q];
+        for (int j = 0; j < Q; ++j) g[j] = f[size_t(j) * n + i], e[j] = g[j];
+        Mom<quad> m;
+        forward(e, m);
+        const quad rho = 1 + m.rho, w = (rho - quad(b.rho_ref)) / 2, T0 = (quad(p.E0) + 28) / 26;
+        const quad pd = (m.E + 28 * m.rho) / 26 - (m.jx * m.jx + m.jy * m.jy) / (2 * rho) - quad(b.heat) / 2;
+        const quad x[8] = {m.rho, m.E, m.jx, m.jy, (m.jx - w * quad(b.gx)) / rho, (m.jy - w * quad(b.gy)) / rho,
+                           (pd - T0 * m.rho) / rho, pd};
+        Mom<double> d;
+        forward(g, d);
+        const double r = 1.0 + d.rho, h = 0.5 * (r - b.rho_ref), t0 = (p.E0 + 28) / 26;
+        const double dp = (d.E + 28.0 * d.rho) / 26.0 - (d.jx * d.jx + d.jy * d.jy) / (2.0 * r) - 0.5 * b.heat;
+        const double y[8] = {d.rho, d.E, d.jx, d.jy, (d.jx - h * b.gx) / r, (d.jy - h * b.gy) / r, (dp - t0 * d.rho) / r, dp};
+        const NodeDev o = node_dev(a, i);
+        const double z[8] = {o.rho, o.E, o.jx, o.jy, o.ux, o.uy, o.T, o.p};
+        for (int c = 0; c < 8; ++c) {
+            value[i * 8 + c] = z[c];
+            ei[i * 8 + c] = double(quad(z[c]) - x[c]);
+            ep[i * 8 + c] = double(quad(y[c]) - x[c]);
+        }
+    }
+}
+extern "C" void read64(const lbm13_params *p, const lbm13_boundary *b, int n, const double *f, double *v, double *ei, double *ep)
+{
+    read_all(*p, *b, n, f, v, ei, ep);
+}
+extern "C" void read32(const lbm13_params *p, const lbm13_boundary *b, int n, const float *f, double *v, double *ei, double *ep)
+{
+    read_all(*p, *b, n, f, v, ei, ep);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    if shutil.which("g++") is None or not os.path.exists(os.path.join(CUDA_INC, "cuda_runtime.h")):
+        pytest.skip("needs g++ and the CUDA headers")
+    d = tmp_path_factory.mktemp("read_states")
+    src, so = d / "read.cpp", d / "read.so"
+    src.write_text(SRC)
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-D__noinline__=", "-fPIC", "-shared", "-w", "-I", CSRC, "-I",
+                           CUDA_INC, str(src), "-o", str(so)])
+    return C.CDLL(str(so))
+
+
+BOUNDS = {"plain": W.boundary(), "buoyancy": W.boundary(gy=-3e-5, rho_ref=1.0), "source": W.boundary(gx=2e-6, gy=1e-6, heat=1e-7)}
+PARAMS = {"pstar": lambda: pstar(0.05, 0.71), "high_pr": lambda: P.select(0.3, 1.0)}
+ptr = lambda a: a.ctypes.data_as(C.c_void_p)  # noqa: E731
+rms = lambda e: np.sqrt(np.mean(e ** 2, axis=0))  # noqa: E731
+
+
+def _read(lib, p, b, f, single):
+    """f [n][13] in the storage type: (values, errors, errors of plain FP64), [n][8]."""
+    g = np.ascontiguousarray(f.T.astype(np.float32 if single else np.float64))
+    out = [np.zeros((len(f), 8)) for _ in range(3)]
+    Pp, Bb = lbm13.make_params(p), lbm13.make_boundary(b)
+    (lib.read32 if single else lib.read64)(C.byref(Pp), C.byref(Bb), len(f), ptr(g), *[ptr(o) for o in out])
+    return out
+
+
+def _check_reading(lib, params, sizes, bound, single):
+    p = PARAMS[params]()
+    f = S._states(p, S.SIZES[sizes], 4000, np.random.default_rng(3), 1e-3)
+    v, ei, ep = _read(lib, p, BOUNDS[bound], f, single)
+    # 4000 nodes estimate each rms to 1.1%; a reading's own last rounding is in both
+    assert (rms(ei) <= 1.05 * rms(ep)).all(), rms(ei) / rms(ep)
+
+
+@pytest.mark.parametrize("bound", list(BOUNDS))
+@pytest.mark.parametrize("sizes", list(S.SIZES))
+@pytest.mark.parametrize("params", list(PARAMS))
+def test_fp64_readings_are_no_less_exact_than_fp64_arithmetic(lib, params, sizes, bound):
+    _check_reading(lib, params, sizes, bound, False)
+
+
+def test_fp64_readings_far_from_rest_and_of_bad_nodes(lib):
+    p = pstar(0.05, 0.71)
+    f = 1e-3 * np.random.default_rng(1).standard_normal((6, Q))
+    f[0] = 0.0
+    f[1, 3] = np.nan
+    f[2, 5] = -np.inf
+    f[3, 0] = 1.5           # density 2.5: the quotients divide
+    f[4, 0] = -0.8
+    f[5] *= 1e-200
+    v, ei, ep = _read(lib, p, W.boundary(), f, False)
+    assert (v[0] == 0).all() and np.isnan(v[1]).any() and not np.isfinite(v[2]).all()
+    u = np.ix_([3, 4, 5], [4, 5])  # the velocities (T and p are differences of larger terms)
+    assert (np.abs(ei[u]) <= 2 * np.abs(ep[u]) + 2.0 ** -52 * np.abs(v[u])).all()
