@@ -921,10 +921,10 @@ int lbm13_set_state_device(lbm13_t h, const double *rho, const double *ux, const
     DeviceGuard g(h->device);
     cudaError_t e;
     if (h->precision == LBM13_FP64)
-        e = launch_init<double>(static_cast<double *>(h->buf[h->cur]), h->nx, h->ny, h->pitch, h->plane, h->kd, h->fi, rho,
+        e = launch_init<double>(static_cast<double *>(h->buf[h->cur]), h->nx, h->ny, h->pitch, h->plane, h->fi, rho,
                                 ux, uy, T, h->stream);
     else
-        e = launch_init<float>(static_cast<float *>(h->buf[h->cur]), h->nx, h->ny, h->pitch, h->plane, h->kd, h->fi, rho,
+        e = launch_init<float>(static_cast<float *>(h->buf[h->cur]), h->nx, h->ny, h->pitch, h->plane, h->fi, rho,
                                ux, uy, T, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "init kernel launch");
     h->t = 0;
@@ -970,10 +970,10 @@ int lbm13_set_state(lbm13_t h, const double *rho, const double *ux, const double
         }
         e = h->precision == LBM13_FP64
                 ? launch_init<double>(static_cast<double *>(h->buf[h->cur]) + (long long)y0 * h->pitch, h->nx, y1 - y0,
-                                      h->pitch, h->plane, h->kd, h->fi, stage + off, stage + n + off, stage + 2 * n + off,
+                                      h->pitch, h->plane, h->fi, stage + off, stage + n + off, stage + 2 * n + off,
                                       stage + 3 * n + off, h->stream)
                 : launch_init<float>(static_cast<float *>(h->buf[h->cur]) + (long long)y0 * h->pitch, h->nx, y1 - y0,
-                                     h->pitch, h->plane, h->kd, h->fi, stage + off, stage + n + off, stage + 2 * n + off,
+                                     h->pitch, h->plane, h->fi, stage + off, stage + n + off, stage + 2 * n + off,
                                      stage + 3 * n + off, h->stream);
         if (e != cudaSuccess) rc = cuda_fail(h, e, "init kernel launch");
     }

@@ -16,7 +16,7 @@ namespace {
 // f*_j = f_eq,j(rho, rho u, E) with E = rho (26 T - 28) + 13 rho |u|^2, stored as
 // the deviation from the rest populations.
 template <typename T>
-__global__ void init_kernel(T *f, int nx, int ny, long long pitch, long long plane, const Coef<double> k, const InitFix c,
+__global__ void init_kernel(T *f, int nx, int ny, long long pitch, long long plane, const InitFix c,
                             const double *__restrict__ rho, const double *__restrict__ ux,
                             const double *__restrict__ uy, const double *__restrict__ Tf)
 {
@@ -24,24 +24,11 @@ __global__ void init_kernel(T *f, int nx, int ny, long long pitch, long long pla
     const int y = blockIdx.y;
     if (x >= nx) return;
     const long long i = (long long)y * nx + x;
-    const double r = rho[i], u = ux[i], v = uy[i], t = Tf[i];
     T *p = f + (long long)y * pitch + x;
-    int64_t F[Q];
-    int q;
-    if (fx_equilibrium(r, u, v, t, c, F, q)) {
+    T g[Q];
+    init_node(rho[i], ux[i], uy[i], Tf[i], c, g);
 #pragma unroll
-        for (int j = 0; j < Q; ++j) {
-            T o;
-            fx_store(F[j], q, o);
-            p[(long long)j * plane] = o;
-        }
-        return;
-    }
-    const double dE = r * (26.0 * t - 28.0) - k.E0 + 13.0 * r * (u * u + v * v);
-    double g[Q];
-    equilibrium_dev(r - 1.0, dE, r * u, r * v, k, g);
-#pragma unroll
-    for (int j = 0; j < Q; ++j) p[(long long)j * plane] = T(g[j]);
+    for (int j = 0; j < Q; ++j) p[(long long)j * plane] = g[j];
 }
 
 // -------------------------------------------------------------- moments
@@ -465,12 +452,11 @@ __global__ void __launch_bounds__(kReduceThreads) project_kernel(const ReadArgs<
 } // namespace
 
 template <typename T>
-cudaError_t launch_init(T *f, int nx, int ny, long long pitch, long long plane, const Coef<double> &k,
-                        const InitFix &x, const double *rho, const double *ux, const double *uy, const double *Tf,
-                        cudaStream_t s)
+cudaError_t launch_init(T *f, int nx, int ny, long long pitch, long long plane, const InitFix &x, const double *rho,
+                        const double *ux, const double *uy, const double *Tf, cudaStream_t s)
 {
     dim3 block(128), grid((nx + 127) / 128, ny);
-    init_kernel<T><<<grid, block, 0, s>>>(f, nx, ny, pitch, plane, k, x, rho, ux, uy, Tf);
+    init_kernel<T><<<grid, block, 0, s>>>(f, nx, ny, pitch, plane, x, rho, ux, uy, Tf);
     return cudaGetLastError();
 }
 
@@ -556,12 +542,10 @@ cudaError_t launch_project(const ReadArgs<T> &a, int kx, int ky, double *partial
     return cudaGetLastError();
 }
 
-template cudaError_t launch_init<double>(double *, int, int, long long, long long, const Coef<double> &,
-                                         const InitFix &, const double *, const double *, const double *,
-                                         const double *, cudaStream_t);
-template cudaError_t launch_init<float>(float *, int, int, long long, long long, const Coef<double> &,
-                                        const InitFix &, const double *, const double *, const double *,
-                                        const double *, cudaStream_t);
+template cudaError_t launch_init<double>(double *, int, int, long long, long long, const InitFix &, const double *,
+                                         const double *, const double *, const double *, cudaStream_t);
+template cudaError_t launch_init<float>(float *, int, int, long long, long long, const InitFix &, const double *,
+                                        const double *, const double *, const double *, cudaStream_t);
 template cudaError_t launch_moments<double>(const ReadArgs<double> &, double *, unsigned, cudaStream_t);
 template cudaError_t launch_moments<float>(const ReadArgs<float> &, double *, unsigned, cudaStream_t);
 template cudaError_t launch_reduce<double>(const ReduceJob<double> &, cudaStream_t);

@@ -234,6 +234,8 @@ inline void init_fix(const lbm13_params &p, const double *D, InitFix &x)
     x.T0 = (p.E0 + 28.0) / 26.0;
     const real rest = 26 * real(x.T0) - 28;
     x.c0 = double((rest - real(p.E0)) / 16);
+    x.rest = double(rest);
+    x.dE0 = double(rest - real(p.E0));
     // dE / 16 = (26 rho dT + (26 T0 - 28) drho + 13 rho |u|^2) / 16 + c0
     x.z = limb(real(26) / 16);
     x.r = limb(rest / 16);
@@ -245,6 +247,8 @@ inline void init_fix(const lbm13_params &p, const double *D, InitFix &x)
         const real E = ME[s] / 4004 + Meps[s] * real(p.c_epsE) / 42196 + Mvpi[s] * real(p.c_vpi_E) / 548;
         x.eR[s] = limb(R);
         x.eE[s] = limb(16 * E);
+        x.R[s] = double(R);
+        x.E[s] = double(E);
         top = std::max(top, std::fabs(R) + std::fabs(16 * E) * 4);
     }
     // unit and distance-2 links per unit of momentum: 1/14 - Q/10 + 2 R/35, 1/7 + Q/10 + R/70
@@ -253,6 +257,14 @@ inline void init_fix(const lbm13_params &p, const double *D, InitFix &x)
     const real A10 = real(1) / 14 - Q0 / 10 + 2 * R0 / 35, A90 = real(1) / 7 + Q0 / 10 + R0 / 70;
     const real a1R = -h1 / 10 + 2 * h2 / 35, a1E = 16 * (-k1 / 10 + 2 * k2 / 35), a9R = h1 / 10 + h2 / 70,
                a9E = 16 * (k1 / 10 + k2 / 70);
+    x.d10 = double(A10);
+    x.l10 = double(A10 - real(x.d10));
+    x.d1R = double(a1R);
+    x.d1E = double(a1E / 16);
+    x.d90 = double(A90);
+    x.l90 = double(A90 - real(x.d90));
+    x.d9R = double(a9R);
+    x.d9E = double(a9E / 16);
     x.a1R = limb(a1R);
     x.a1E = limb(a1E);
     x.a9R = limb(a9R);

@@ -130,7 +130,7 @@ struct ReadArgs {
     double gx, gy, rho_ref;
     double heat;  // energy source q: T is read half-way, (p* - q/2)/rho
     int force;    // nonzero when g != 0
-    ReadFix fx;   // the same in integers
+    ReadFix fx;   // the constants in integers (FP32 storage)
 };
 
 // Streaming multiprocessors of the current device (queried once per device;
@@ -158,8 +158,8 @@ cudaError_t launch_halo(T *f, int nx, int ny, long long pitch, long long plane, 
                         cudaStream_t s);
 
 template <typename T>
-cudaError_t launch_init(T *f, int nx, int ny, long long pitch, long long plane, const Coef<double> &k,
-                        const InitFix &x, const double *rho, const double *ux, const double *uy, const double *Tf, cudaStream_t s);
+cudaError_t launch_init(T *f, int nx, int ny, long long pitch, long long plane, const InitFix &x, const double *rho,
+                        const double *ux, const double *uy, const double *Tf, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_moments(const ReadArgs<T> &a, double *out, unsigned mask, cudaStream_t s);

@@ -1,6 +1,7 @@
-"""Read-outs (csrc/lbm13_read.cuh) on the host, at the states that flows hold: a small velocity beside large deviations of
+"""Read-outs and initial states (csrc/lbm13_read.cuh, csrc/lbm13_fixed_io.cuh) on the
+host, at the states that flows hold: a small velocity beside large deviations of
 density and temperature, and the other way round.  Against 113-bit arithmetic no
-reading is less exact than FP64 arithmetic with one rounding per
+reading and no momentum is less exact than FP64 arithmetic with one rounding per
 operation gives it."""
 import ctypes as C
 import os
@@ -143,3 +144,73 @@ def test_fp64_readings_far_from_rest_and_of_bad_nodes(lib):
     assert (v[0] == 0).all() and np.isnan(v[1]).any() and not np.isfinite(v[2]).all()
     u = np.ix_([3, 4, 5], [4, 5])  # the velocities (T and p are differences of larger terms)
     assert (np.abs(ei[u]) <= 2 * np.abs(ep[u]) + 2.0 ** -52 * np.abs(v[u])).all()
+
+
+INIT_SRC = r"""
+// in [n][4]: rho, ux, uy, T; errors [n][17] of the 13 deviations, j_x, j_y, E and f1 - f3
+extern "C" void init64(const lbm13_params *p, const double *D, const lbm13_boundary *b, int n, const double *in, double *ei,
+                       double *ep)
+{
+    Coef<double> kd;
+    collision_coef(*p, D, *b, kd);
+    InitFix k;
+    init_fix(*p, D, k);
+    for (int i = 0; i < n; ++i) {
+        const double r = in[4 * i], u = in[4 * i + 1], v = in[4 * i + 2], t = in[4 * i + 3];
+        const quad R = quad(r) - 1, jx = quad(r) * u, jy = quad(r) * v;
+        const quad dE = quad(r) * (26 * quad(t) - 28) - quad(p->E0) + 13 * quad(r) * (quad(u) * u + quad(v) * v);
+        const quad Qe = quad(p->c1) + quad(D[2]) * (1 + R) + quad(D[3]) * (quad(p->E0) + dE);
+        const quad Re = quad(D[5]) + quad(D[4]) * (1 + R) + quad(p->k2) * (quad(p->E0) + dE);
+        Mom<quad> d;
+        d.rho = R / 13;
+        d.E = dE / 4004;
+        d.eps = (quad(D[6]) * R + quad(p->c_epsE) * dE) / 42196;
+        d.vpi = (quad(p->c_vpi_rho) * R + quad(p->c_vpi_E) * dE) / 548;
+        d.jx = jx / 14;
+        d.jy = jy / 14;
+        d.qx = jx * Qe / 20;
+        d.qy = jy * Qe / 20;
+        d.rx = jx * Re / 70;
+        d.ry = jy * Re / 70;
+        d.XX = (jx * jx - jy * jy) / quad(r) / 68;
+        d.XY = jx * jy / quad(r) / 4;
+        d.XXe = 0;
+        quad e[Q] = {};
+        inverse_add<true>(d, e);
+        double g[2][Q];
+        init_node(r, u, v, t, k, g[0]);
+        equilibrium_dev(r - 1.0, r * (26.0 * t - 28.0) - p->E0 + 13.0 * r * (u * u + v * v), r * u, r * v, kd, g[1]);
+        for (int w = 0; w < 2; ++w) {
+            double *o = (w ? ep : ei) + i * 17;
+            quad q[Q];
+            Mom<quad> m;
+            for (int j = 0; j < Q; ++j) q[j] = g[w][j], o[j] = double(q[j] - e[j]);
+            forward(q, m);
+            o[13] = double(m.jx - jx);
+            o[14] = double(m.jy - jy);
+            o[15] = double(m.E - dE);
+            o[16] = double((q[1] - q[3]) - (e[1] - e[3]));
+        }
+    }
+}
+"""
+
+
+@pytest.mark.parametrize("sizes", list(S.SIZES))
+@pytest.mark.parametrize("params", list(PARAMS))
+def test_fp64_initial_states_are_no_less_exact_than_fp64_arithmetic(tmp_path, params, sizes):
+    if shutil.which("g++") is None or not os.path.exists(os.path.join(CUDA_INC, "cuda_runtime.h")):
+        pytest.skip("needs g++ and the CUDA headers")
+    src, so = tmp_path / "init.cpp", tmp_path / "init.so"
+    src.write_text(SRC + INIT_SRC)
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-D__noinline__=", "-fPIC", "-shared", "-w", "-I",
+                           CSRC, "-I", CUDA_INC, str(src), "-o", str(so)])
+    p = PARAMS[params]()
+    st, D = lbm13.lbm13_derive(p)
+    n, a = 4000, S.SIZES[sizes]
+    x = np.array([1.0, 0.0, 0.0, P.rest_temperature(p)]) + np.array([a[0], a[1], a[1], a[2]]) * np.random.default_rng(5).standard_normal((n, 4))
+    x = np.ascontiguousarray(x)
+    ei, ep = np.zeros((n, 17)), np.zeros((n, 17))
+    Pp, Bb = lbm13.make_params(p), lbm13.make_boundary(W.boundary())
+    C.CDLL(str(so)).init64(C.byref(Pp), ptr(np.ascontiguousarray(D)), C.byref(Bb), n, ptr(x), ptr(ei), ptr(ep))
+    assert (rms(ei) <= 1.05 * rms(ep)).all(), rms(ei) / rms(ep)
