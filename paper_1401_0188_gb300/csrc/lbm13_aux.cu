@@ -106,13 +106,13 @@ __device__ __forceinline__ void put_fields_fixed(const ReadArgs<float> &a, const
     if (mask & 0x400u) put(s.value(s.X1 + 4 * s.X9));
     if (mask & 0x800u) put(s.value(s.X5));
     if (mask & 0x1000u) put(s.value(s.X9 - 4 * s.X1));
-    if (mask & 0x2000u) put(s.value(m.ux));
-    if (mask & 0x4000u) put(s.value(m.uy));
+    if (mask & 0x2000u) put(s.value(m.u));
+    if (mask & 0x4000u) put(s.value(m.v));
     const double T0 = a.rest.T0;
-    if (mask & 0x8000u) put(T0 + s.value(m.dT));
-    if (mask & 0x10000u) put(T0 + s.value(m.dp));
+    if (mask & 0x8000u) put(T0 + s.value(m.T));
+    if (mask & 0x10000u) put(T0 + s.value(m.p));
     if (mask & 0x20000u) {
-        const double ux = s.value(m.ux), uy = s.value(m.uy);
+        const double ux = s.value(m.u), uy = s.value(m.v);
         put(a.rest.E0 + s.energy() - 6.5 * (ux * ux + uy * uy));
     }
 }

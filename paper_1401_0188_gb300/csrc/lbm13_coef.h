@@ -214,8 +214,13 @@ inline void read_fix(double E0, const lbm13_boundary &b, ReadFix &x)
     const auto limb = [](double c) { return fx_coef(int64_t(std::llrint(std::ldexp(c, 57)))); };
     x.on = 1;
     x.T0 = limb(T0);
-    x.hgx = limb(0.5 * b.gx);
-    x.hgy = limb(0.5 * b.gy);
+    const auto scaled = [&](double c, int &e) {
+        std::frexp(c, &e);  // |c| < 2^e
+        e = c == 0.0 ? 0 : std::min(std::max(-1 - e, 0), 60);
+        return limb(std::ldexp(c, e));
+    };
+    x.hgx = scaled(0.5 * b.gx, x.ex);
+    x.hgy = scaled(0.5 * b.gy, x.ey);
     x.Fx0 = 0.5 * (1.0 - b.rho_ref) * b.gx;
     x.Fy0 = 0.5 * (1.0 - b.rho_ref) * b.gy;
     x.half_q = 0.5 * b.heat;

@@ -137,10 +137,10 @@ __device__ __forceinline__ NodeDev node_dev(const ReadArgs<float> &a, long long 
     o.E = s.energy();
     o.jx = s.value(s.jx());
     o.jy = s.value(s.jy());
-    o.ux = s.value(m.ux);
-    o.uy = s.value(m.uy);
-    o.T = s.value(m.dT);
-    o.p = s.value(m.dp);
+    o.ux = s.value(m.u);
+    o.uy = s.value(m.v);
+    o.T = s.value(m.T);
+    o.p = s.value(m.p);
     o.bad = 0.0;
     return o;
 }

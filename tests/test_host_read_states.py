@@ -214,3 +214,78 @@ def test_fp64_initial_states_are_no_less_exact_than_fp64_arithmetic(tmp_path, pa
     Pp, Bb = lbm13.make_params(p), lbm13.make_boundary(W.boundary())
     C.CDLL(str(so)).init64(C.byref(Pp), ptr(np.ascontiguousarray(D)), C.byref(Bb), n, ptr(x), ptr(ei), ptr(ep))
     assert (rms(ei) <= 1.05 * rms(ep)).all(), rms(ei) / rms(ep)
+
+
+@pytest.mark.parametrize("bound", list(BOUNDS))
+@pytest.mark.parametrize("sizes", list(S.SIZES))
+@pytest.mark.parametrize("params", list(PARAMS))
+def test_fp32_readings_are_no_less_exact_than_fp64_arithmetic(lib, params, sizes, bound):
+    _check_reading(lib, params, sizes, bound, True)
+
+
+def test_fp32_readings_of_floats_below_the_normal_range(lib):
+    """Nodes of 1e-30 and less, some of whose populations are subnormal."""
+    p = pstar(0.05, 0.71)
+    rng = np.random.default_rng(8)
+    f = rng.standard_normal((2000, Q)) * 10.0 ** rng.integers(-36, -18, (2000, 1)).astype(float)
+    f[:, 3:9] *= 1e-7
+    v, ei, ep = _read(lib, p, W.boundary(), f, True)
+    scale = np.abs(f).max(axis=1)[:, None]
+    assert (rms(ei / scale) <= 1.05 * rms(ep / scale)).all()
+
+
+@pytest.mark.parametrize("mirror", list(S.MIRRORS))
+@pytest.mark.parametrize("bound", list(BOUNDS))
+@pytest.mark.parametrize("single", [False, True])
+def test_mirrored_nodes_read_to_mirrored_values(lib, single, bound, mirror):
+    p, b, m = pstar(0.05, 0.71), BOUNDS[bound], S.MIRRORS[mirror]
+    image = dict(b, gx=b["gx"] * (-1 if "x" in mirror else 1), gy=b["gy"] * (-1 if "y" in mirror else 1))
+    f = np.concatenate([S._states(p, a, 2000, np.random.default_rng(9), 1e-3) for a in S.SIZES.values()])
+    sign = np.ones(8)
+    sign[[2, 4]] *= -1 if "x" in mirror else 1
+    sign[[3, 5]] *= -1 if "y" in mirror else 1
+    assert np.array_equal(_read(lib, p, b, f, single)[0] * sign, _read(lib, p, image, f[:, m], single)[0])
+
+
+MIRROR_SRC = r"""
+template <typename T>
+static void init_all(const lbm13_params &p, const double *D, int n, const double *in, T *out)
+{
+    InitFix k;
+    init_fix(p, D, k);
+    for (int i = 0; i < n; ++i) {
+        T g[Q];
+        init_node(in[4 * i], in[4 * i + 1], in[4 * i + 2], in[4 * i + 3], k, g);
+        for (int j = 0; j < Q; ++j) out[i * Q + j] = g[j];
+    }
+}
+extern "C" void set64(const lbm13_params *p, const double *D, int n, const double *in, double *out) { init_all(*p, D, n, in, out); }
+extern "C" void set32(const lbm13_params *p, const double *D, int n, const double *in, float *out) { init_all(*p, D, n, in, out); }
+"""
+
+
+@pytest.mark.parametrize("single", [False, True])
+def test_mirrored_initial_states_are_mirror_images(tmp_path, single):
+    if shutil.which("g++") is None or not os.path.exists(os.path.join(CUDA_INC, "cuda_runtime.h")):
+        pytest.skip("needs g++ and the CUDA headers")
+    src, so = tmp_path / "set.cpp", tmp_path / "set.so"
+    src.write_text(SRC + MIRROR_SRC)
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-D__noinline__=", "-fPIC", "-shared", "-w", "-I",
+                           CSRC, "-I", CUDA_INC, str(src), "-o", str(so)])
+    L, p = C.CDLL(str(so)), pstar(0.05, 0.71)
+    st, D = lbm13.lbm13_derive(p)
+    n, dtype = 20000, np.float32 if single else np.float64
+    rng = np.random.default_rng(6)
+    x = np.array([1.0, 0.0, 0.0, P.rest_temperature(p)]) + 10.0 ** rng.integers(-5, -1, (n, 1)).astype(float) * rng.standard_normal((n, 4))
+    x[::2, 1:3] = np.round(x[::2, 1:3] * 2.0 ** 12) * 2.0 ** -12  # few significant bits
+    Pp = lbm13.make_params(p)
+
+    def state(y):
+        out = np.zeros((n, Q), dtype=dtype)
+        (L.set32 if single else L.set64)(C.byref(Pp), ptr(np.ascontiguousarray(D)), n, ptr(np.ascontiguousarray(y)), ptr(out))
+        return out
+
+    f = state(x)
+    for mirror, m in S.MIRRORS.items():
+        sign = np.array([1.0, -1.0 if "x" in mirror else 1.0, -1.0 if "y" in mirror else 1.0, 1.0])
+        assert np.array_equal(f[:, m], state(x * sign))
