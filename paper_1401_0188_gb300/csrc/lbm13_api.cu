@@ -161,6 +161,21 @@ void dev_free(lbm13_t h, void *p, size_t bytes)
     h->bytes_held -= bytes < h->bytes_held ? bytes : h->bytes_held;
 }
 
+// Memory with bytes [from, from + len) zeroed on stream s.  Nothing is kept of
+// memory that could not be cleared (what: for the message).
+int dev_zeroed(lbm13_t h, void *&p, size_t bytes, size_t from, size_t len, cudaStream_t s, const char *what)
+{
+    void *m = dev_alloc(h, bytes);
+    if (!m) return fail(h, LBM13_ENOMEM, std::string("allocator returned NULL for ") + what);
+    const cudaError_t e = cudaMemsetAsync(static_cast<char *>(m) + from, 0, len, s);
+    if (e != cudaSuccess) {
+        dev_free(h, m, bytes);
+        return cuda_fail(h, e, what);
+    }
+    p = m;
+    return LBM13_OK;
+}
+
 bool finite_all(std::initializer_list<double> v)
 {
     for (double x : v)
@@ -346,12 +361,10 @@ GridSync grid_sync(lbm13_t h)
 }
 
 // The step launches' error word and grid-barrier words (made on first use).
-bool ensure_sync_mem(lbm13_t h)
+int ensure_sync_mem(lbm13_t h)
 {
-    if (h->sync_mem) return true;
-    h->sync_mem = dev_alloc(h, kSyncBytes);
-    if (!h->sync_mem) return false;
-    return cudaMemsetAsync(h->sync_mem, 0, kSyncBytes, h->stream) == cudaSuccess;
+    if (h->sync_mem) return LBM13_OK;
+    return dev_zeroed(h, h->sync_mem, kSyncBytes, 0, kSyncBytes, h->stream, "the step error word");
 }
 
 // Whether lbm13_step takes n steps from shared memory (resident_kernel): where a
@@ -385,15 +398,14 @@ bool use_resident(lbm13_t h, long long n)
         cudaGetLastError();
         return false;
     }
-    if (!ensure_sync_mem(h)) return false;
+    if (ensure_sync_mem(h) != LBM13_OK) return false;
     if (!h->res_xchg) {
         const size_t bytes = res_exchange_bytes(h->nx, h->ny, int(h->elem));
-        h->res_xchg = dev_alloc(h, bytes);
-        if (!h->res_xchg) {  // no memory for it: step launch by launch from here on
-            h->res.ex = 0;
+        if (dev_zeroed(h, h->res_xchg, bytes, 0, bytes, h->stream, "the exchange buffer") != LBM13_OK) {
+            cudaGetLastError();
+            h->res.ex = 0;  // step launch by launch from here on
             return false;
         }
-        if (cudaMemsetAsync(h->res_xchg, 0, bytes, h->stream) != cudaSuccess) return false;
         h->res_tag = 0;
     }
     return true;
@@ -405,7 +417,7 @@ bool use_persistent(lbm13_t h, long long n)
     if (h->persistent != LBM13_PERSISTENT_ON || n < 2) return false;
     if (h->multi_grid < 0) h->multi_grid = multi_grid<T, C>(h->nx, h->ny, h->force);
     if (h->multi_grid <= 0) return false;
-    return ensure_sync_mem(h);
+    return ensure_sync_mem(h) == LBM13_OK;
 }
 
 // Reports (and clears) a grid-barrier timeout of an earlier persistent launch;
@@ -470,7 +482,7 @@ cudaError_t build_pair_graph(lbm13_t h, int cur)
 // for an odd remainder.
 int do_pair_steps(lbm13_t h, long long n)
 {
-    if (!ensure_sync_mem(h)) return fail(h, LBM13_ENOMEM, "allocator returned NULL for the step error word");
+    if (const int rc = ensure_sync_mem(h)) return rc;
     if (n >= kGraphSteps) {
         if (!h->gexec2[h->cur]) {
             cudaError_t e = build_pair_graph(h, h->cur);
@@ -601,8 +613,11 @@ int ensure_reduce(lbm13_t h, cudaStream_t s)
     const long long n = (long long)h->nx * h->ny;
     const int nb = reduce_blocks(h->nx, h->ny);
     const size_t doubles = size_t(6 * n) + size_t(nb) * kPartials + kReduceTail;
-    h->red_mem = dev_alloc(h, doubles * sizeof(double));
-    if (!h->red_mem) return fail(h, LBM13_ENOMEM, "allocator returned NULL for the reduction buffers");
+    // the count of finished blocks, the last double, starts at zero (and is left so by
+    // every pass)
+    if (const int rc = dev_zeroed(h, h->red_mem, doubles * sizeof(double), (doubles - 1) * sizeof(double), sizeof(double), s,
+                                  "the reduction buffers"))
+        return rc;
     double *base = static_cast<double *>(h->red_mem);
     h->rb.fields = base;
     h->rb.snap = base + 3 * n;
@@ -611,9 +626,6 @@ int ensure_reduce(lbm13_t h, cudaStream_t s)
     h->rb.nblocks = nb;
     h->out_dev = h->rb.stats + 16;
     h->rb.done = reinterpret_cast<unsigned *>(h->out_dev + 17);
-    // counts of finished blocks start at zero (and are left so by every pass)
-    cudaError_t e = cudaMemsetAsync(h->rb.done, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return cuda_fail(h, e, "reduction set-up");
     return LBM13_OK;
 }
 
@@ -869,7 +881,7 @@ int lbm13_pair_check(lbm13_t h, double timeout_s, int withhold, int *timed_out)
         return fail(h, LBM13_EINVAL, "NULL argument or timeout_s outside [1e-3, 2]");
     DeviceGuard g(h->device);
     if (!use_pairs(h)) return fail(h, LBM13_EINVAL, "the lattice does not take paired steps");
-    if (!ensure_sync_mem(h)) return fail(h, LBM13_ENOMEM, "allocator returned NULL for the step error word");
+    if (const int rc = ensure_sync_mem(h)) return rc;
     CK(h, cudaStreamSynchronize(h->stream));
     int rc = check_barrier_error(h);
     if (rc != LBM13_OK) return rc;
@@ -1164,10 +1176,11 @@ int lbm13_project(lbm13_t h, int kx, int ky, double *out)
     DeviceGuard g(h->device);
     if (!h->proj_mem) {
         const int nb = reduce_blocks(h->nx, h->ny);
-        h->proj_mem = dev_alloc(h, (size_t(nb + 1) * kProj + 1) * sizeof(double));
-        if (!h->proj_mem) return fail(h, LBM13_ENOMEM, "allocator returned NULL for the projection buffers");
+        const size_t count = size_t(nb + 1) * kProj * sizeof(double);  // before the block count
+        if (const int rc = dev_zeroed(h, h->proj_mem, count + sizeof(double), count, sizeof(double), h->stream,
+                                      "the projection buffers"))
+            return rc;
         h->proj_blocks = nb;
-        CK(h, cudaMemsetAsync(static_cast<double *>(h->proj_mem) + size_t(nb + 1) * kProj, 0, sizeof(double), h->stream));
     }
     double *partials = static_cast<double *>(h->proj_mem);
     double *res = partials + size_t(h->proj_blocks) * kProj;
@@ -1452,7 +1465,11 @@ int plan_upload_maps(lbm13_plan_t p)
         p->tma_err = static_cast<unsigned *>(plan_alloc(p, sizeof(unsigned)));
         if (!p->tma_err) return pfail(p, LBM13_ENOMEM, "allocator returned NULL for the plan's error word");
         cudaError_t e = cudaMemsetAsync(p->tma_err, 0, sizeof(unsigned), p->stream);
-        if (e != cudaSuccess) return pfail(p, LBM13_ECUDA, std::string("plan error word: ") + cudaGetErrorString(e));
+        if (e != cudaSuccess) {
+            plan_free(p, p->tma_err);
+            p->tma_err = nullptr;
+            return pfail(p, LBM13_ECUDA, std::string("plan error word: ") + cudaGetErrorString(e));
+        }
     }
     // pageable source: staged before the call returns, ordered on the plan's stream
     cudaError_t e = cudaMemcpyAsync(p->maps, host.data(), bytes, cudaMemcpyHostToDevice, p->stream);
