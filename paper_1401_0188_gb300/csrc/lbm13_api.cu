@@ -138,13 +138,24 @@ struct DeviceGuard {
     }
 };
 
+// cudaMalloc that neither fails for nor breaks a graph capture under way elsewhere in
+// the process (stepping allocates on first use).
+cudaError_t malloc_relaxed(void **p, size_t bytes)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    const bool swapped = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (swapped) cudaThreadExchangeStreamCaptureMode(&mode);
+    return e;
+}
+
 void *dev_alloc(lbm13_t h, size_t bytes)
 {
     bytes = (bytes + 255) & ~size_t(255);
     void *p = nullptr;
     if (h->has_alloc) {
         p = h->alloc.alloc(bytes, h->alloc.ctx);
-    } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    } else if (malloc_relaxed(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
         p = nullptr;
     }
@@ -374,7 +385,7 @@ int ensure_sync_mem(lbm13_t h)
 // keeps the launches it would have recorded before.
 constexpr long long kResMinSteps = 32;
 
-bool use_resident(lbm13_t h, long long n)
+bool wants_resident(lbm13_t h, long long n)
 {
     if (h->persistent == LBM13_PERSISTENT_OFF || n < (h->persistent == LBM13_PERSISTENT_ON ? 2 : kResMinSteps) ||
         h->b.south.kind == HALO || h->b.north.kind == HALO)
@@ -387,6 +398,11 @@ bool use_resident(lbm13_t h, long long n)
         h->res = coop ? res_shape(h->nx, h->ny, h->b.west.kind == PERIODIC, h->b.south.kind == PERIODIC, int(h->elem),
                                   device_sm_count())
                       : ResShape{0, 0, 0, 0, 0, 0, 0};
+        // all tiles at once, as the device is shared out to this process
+        if (h->res.ex && h->res.gx * h->res.gy > (h->precision == LBM13_FP64
+                                                      ? resident_capacity<double, double>(h->res, h->force, h->wd)
+                                                      : resident_capacity<float, float>(h->res, h->force, h->wf)))
+            h->res.ex = 0;
     }
     if (h->res.ex == 0) return false;
     // memory from an allocator of the caller's is ordered on the stream the
@@ -398,7 +414,13 @@ bool use_resident(lbm13_t h, long long n)
         cudaGetLastError();
         return false;
     }
-    if (ensure_sync_mem(h) != LBM13_OK) return false;
+    return true;
+}
+
+// The same with its exchange buffer made, on first use.
+bool use_resident(lbm13_t h, long long n)
+{
+    if (!wants_resident(h, n) || ensure_sync_mem(h) != LBM13_OK) return false;
     if (!h->res_xchg) {
         const size_t bytes = res_exchange_bytes(h->nx, h->ny, int(h->elem));
         if (dev_zeroed(h, h->res_xchg, bytes, 0, bytes, h->stream, "the exchange buffer") != LBM13_OK) {
@@ -412,12 +434,16 @@ bool use_resident(lbm13_t h, long long n)
 }
 
 template <typename T, typename C>
-bool use_persistent(lbm13_t h, long long n)
+bool wants_persistent(lbm13_t h, long long n)
 {
     if (h->persistent != LBM13_PERSISTENT_ON || n < 2) return false;
     if (h->multi_grid < 0) h->multi_grid = multi_grid<T, C>(h->nx, h->ny, h->force);
-    if (h->multi_grid <= 0) return false;
-    return ensure_sync_mem(h) == LBM13_OK;
+    return h->multi_grid > 0;
+}
+template <typename T, typename C>
+bool use_persistent(lbm13_t h, long long n)
+{
+    return wants_persistent<T, C>(h, n) && ensure_sync_mem(h) == LBM13_OK;
 }
 
 // Reports (and clears) a grid-barrier timeout of an earlier persistent launch;
@@ -524,14 +550,20 @@ int do_steps(lbm13_t h, long long n, const Coef<C> &k, const WallArgs<C> *w)
             }
             cudaError_t e = launch_resident<T, C>(step_args<T, C>(h, h->cur, k, w), h->force, m, h->res, h->res_xchg,
                                                   h->res_tag, step_err(h), kBarrierTimeoutNs, h->stream);
-            if (e != cudaSuccess) return cuda_fail(h, e, "resident step launch");
+            if (e != cudaSuccess) {
+                // refused (the SMs that this process may use have become fewer, say): the
+                // remaining steps are other launches, which report what stands against any
+                cudaGetLastError();
+                h->res.ex = 0;
+                break;
+            }
             if (h->persistent == LBM13_PERSISTENT_ON) h->shown_grid = h->res.gx * h->res.gy;
             h->res_tag += unsigned(x);
             h->cur ^= m & 1;
             h->t += m;
             n -= m;
         }
-        return LBM13_OK;
+        if (n == 0) return LBM13_OK;
     }
     if (use_persistent<T, C>(h, n)) {
         const GridSync g = grid_sync(h);
@@ -856,10 +888,9 @@ int lbm13_step_launches(lbm13_t h, int64_t n, int64_t *launches)
     DeviceGuard g(h->device);
     if (n >= 2 && h->precision != LBM13_FP64 && use_pairs(h))
         *launches = n / 2 + (n & 1);
-    else if (use_resident(h, n))
+    else if (wants_resident(h, n))
         *launches = (n + kPersistentChunk - 1) / kPersistentChunk;
-    else if (n >= 2 && (h->precision == LBM13_FP64 ? use_persistent<double, double>(h, n)
-                                                     : use_persistent<float, float>(h, n)))
+    else if (h->precision == LBM13_FP64 ? wants_persistent<double, double>(h, n) : wants_persistent<float, float>(h, n))
         *launches = (n + kPersistentChunk - 1) / kPersistentChunk;
     else
         *launches = n;
@@ -1340,7 +1371,7 @@ void *plan_alloc(lbm13_plan_t p, size_t bytes)
     bytes = (bytes + 255) & ~size_t(255);
     void *ptr = nullptr;
     if (p->has_alloc) ptr = p->alloc.alloc(bytes, p->alloc.ctx);
-    else if (cudaMalloc(&ptr, bytes) != cudaSuccess) { cudaGetLastError(); ptr = nullptr; }
+    else if (malloc_relaxed(&ptr, bytes) != cudaSuccess) { cudaGetLastError(); ptr = nullptr; }
     return ptr;
 }
 
@@ -1703,6 +1734,7 @@ int plan_setup_resident(lbm13_plan_t p)
         p->res_smem_bytes = std::max(p->res_smem_bytes, res_smem(s, 4));
     }
     p->res_ntiles = int(tiles.size());
+    if (p->res_ntiles > resident_plan_capacity(p->res_ex, p->res_threads, p->res_smem_bytes, p->res_states)) return LBM13_OK;
     const size_t table = tiles.size() * sizeof(ResPlanTile);
     if (!plan_room(p, p->res_xchg, p->res_xchg_bytes, bytes) || !plan_room(p, p->res_tiles, p->res_tiles_bytes, table))
         return LBM13_OK;
@@ -1735,7 +1767,9 @@ int plan_use_resident(lbm13_plan_t p, long long n, bool &use)
     return rc;
 }
 
-int plan_steps_resident(lbm13_plan_t p, long long n)
+// Takes n steps so and leaves in n those that a refused launch did not take (see
+// do_steps): the plan then steps launch by launch until its lattices change.
+int plan_steps_resident(lbm13_plan_t p, long long &n)
 {
     while (n > 0) {
         const int m = int(n < kPersistentChunk ? n : kPersistentChunk);
@@ -1749,7 +1783,11 @@ int plan_steps_resident(lbm13_plan_t p, long long n)
                                              static_cast<const ResPlanTile *>(p->res_tiles), p->res_ntiles, p->res_ex,
                                              p->res_threads, p->res_smem_bytes, p->res_states, p->parity, m,
                                              p->res_xchg, p->res_tag, p->tma_err, kBarrierTimeoutNs, p->stream);
-        if (e != cudaSuccess) return pfail(p, LBM13_ECUDA, std::string("resident plan launch: ") + cudaGetErrorString(e));
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            p->res_ready = 0;
+            return LBM13_OK;
+        }
         p->res_tag += x;
         plan_advance(p, m);
         n -= m;
@@ -1764,7 +1802,7 @@ int plan_steps(lbm13_plan_t p, long long n, bool tuning = false)
     bool resident = false;
     if (!tuning) rc = plan_use_resident(p, n, resident);
     if (rc != LBM13_OK) return rc;
-    if (resident) return plan_steps_resident(p, n);
+    if (resident && ((rc = plan_steps_resident(p, n)) != LBM13_OK || n == 0)) return rc;
     if (n >= kGraphSteps) {
         if (!p->gexec[p->parity]) {
             cudaError_t e = cudaSuccess;

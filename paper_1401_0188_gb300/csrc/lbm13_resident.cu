@@ -409,17 +409,44 @@ const void *resident_fn(int ex, bool force)
                  : reinterpret_cast<const void *>(&resident_kernel<T, C, false, 48, States>);
 }
 
+// The kernel of a split, its allowance raised.
+template <typename T, typename C>
+cudaError_t resident_ready(const ResShape &s, bool force, bool states, const void *&fn)
+{
+    fn = states ? resident_fn<T, C, true>(s.ex, force) : resident_fn<T, C, false>(s.ex, force);
+    static std::atomic<unsigned long long> raised[4 * kResWidths];
+    const int which = (s.ex == 24 ? 0 : s.ex == 32 ? 1 : 2) + (force ? kResWidths : 0) + (states ? 2 * kResWidths : 0);
+    return res_allow(fn, raised[which]);
+}
+cudaError_t resident_plan_ready(int ex, bool states, const void *&fn)
+{
+    const bool wide = ex == kResPlanWidths[1];
+    fn = wide ? (states ? reinterpret_cast<const void *>(&resident_plan_kernel<kResPlanWidths[1], true>)
+                        : reinterpret_cast<const void *>(&resident_plan_kernel<kResPlanWidths[1], false>))
+              : (states ? reinterpret_cast<const void *>(&resident_plan_kernel<kResPlanWidths[0], true>)
+                        : reinterpret_cast<const void *>(&resident_plan_kernel<kResPlanWidths[0], false>));
+    static std::atomic<unsigned long long> raised[4];
+    return res_allow(fn, raised[(wide ? 2 : 0) + (states ? 1 : 0)]);
+}
+
+int res_capacity(const void *fn, int threads, size_t smem)
+{
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return per * device_sm_count();
+}
+
 } // namespace
 
 template <typename T, typename C>
 cudaError_t launch_resident(const StepArgs<T, C> &a, bool force, int nsteps, const ResShape &s, void *xchg,
                             unsigned tag, unsigned *err, unsigned long long timeout_ns, cudaStream_t stream)
 {
-    const bool states = res_states_pass(a.wall);
-    const void *fn = states ? resident_fn<T, C, true>(s.ex, force) : resident_fn<T, C, false>(s.ex, force);
-    static std::atomic<unsigned long long> raised[4 * kResWidths];
-    const int which = (s.ex == 24 ? 0 : s.ex == 32 ? 1 : 2) + (force ? kResWidths : 0) + (states ? 2 * kResWidths : 0);
-    const cudaError_t e = res_allow(fn, raised[which]);
+    const void *fn = nullptr;
+    const cudaError_t e = resident_ready<T, C>(s, force, res_states_pass(a.wall), fn);
     if (e != cudaSuccess) return e;
     StepArgs<T, C> pa = a;
     if (nsteps % 2 == 0) pa.fout = const_cast<T *>(a.fin);
@@ -430,23 +457,40 @@ cudaError_t launch_resident(const StepArgs<T, C> &a, bool force, int nsteps, con
                                        res_smem(s, int(sizeof(T))), stream);
 }
 
+template <typename T, typename C>
+int resident_capacity(const ResShape &s, bool force, const WallArgs<C> *wall)
+{
+    const void *fn = nullptr;
+    if (resident_ready<T, C>(s, force, res_states_pass(wall), fn) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return res_capacity(fn, s.threads, res_smem(s, int(sizeof(T))));
+}
+int resident_plan_capacity(int ex, int threads, size_t smem, bool states)
+{
+    const void *fn = nullptr;
+    if (resident_plan_ready(ex, states, fn) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return res_capacity(fn, threads, smem);
+}
+
 cudaError_t launch_resident_plan(const BatchDesc<float, float> *descs, const ResPlanTile *tiles, int ntiles, int ex,
                                  int threads, size_t smem, bool states, int parity, int nsteps, void *xchg,
                                  unsigned tag, unsigned *err, unsigned long long timeout_ns, cudaStream_t stream)
 {
-    const bool wide = ex == kResPlanWidths[1];
-    const void *fn = wide ? (states ? reinterpret_cast<const void *>(&resident_plan_kernel<kResPlanWidths[1], true>)
-                                    : reinterpret_cast<const void *>(&resident_plan_kernel<kResPlanWidths[1], false>))
-                          : (states ? reinterpret_cast<const void *>(&resident_plan_kernel<kResPlanWidths[0], true>)
-                                    : reinterpret_cast<const void *>(&resident_plan_kernel<kResPlanWidths[0], false>));
-    static std::atomic<unsigned long long> raised[4];
-    const cudaError_t e = res_allow(fn, raised[(wide ? 2 : 0) + (states ? 1 : 0)]);
+    const void *fn = nullptr;
+    const cudaError_t e = resident_plan_ready(ex, states, fn);
     if (e != cudaSuccess) return e;
     unsigned char *px = static_cast<unsigned char *>(xchg);
     void *args[] = {&descs, &tiles, &parity, &nsteps, &px, &tag, &err, &timeout_ns};
     return cudaLaunchCooperativeKernel(fn, dim3(ntiles), dim3(threads), args, smem, stream);
 }
 
+template int resident_capacity<double, double>(const ResShape &, bool, const WallArgs<double> *);
+template int resident_capacity<float, float>(const ResShape &, bool, const WallArgs<float> *);
 template cudaError_t launch_resident<double, double>(const StepArgs<double, double> &, bool, int, const ResShape &,
                                                      void *, unsigned, unsigned *, unsigned long long, cudaStream_t);
 template cudaError_t launch_resident<float, float>(const StepArgs<float, float> &, bool, int, const ResShape &, void *,

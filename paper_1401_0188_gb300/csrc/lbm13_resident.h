@@ -354,6 +354,10 @@ template <typename T, typename C>
 cudaError_t launch_resident(const StepArgs<T, C> &a, bool force, int nsteps, const ResShape &s, void *xchg,
                             unsigned tag, unsigned *err, unsigned long long timeout_ns, cudaStream_t stream);
 
+// Blocks of such a launch that the SMs hold at once (0 where it cannot be launched).
+template <typename T, typename C>
+int resident_capacity(const ResShape &s, bool force, const WallArgs<C> *wall);
+
 // The same for the lattices of a plan, block i stepping tile[i].  All shapes have
 // rows of `ex` columns (kResPlanWidths); xchg holds the lattices' exchange buffers
 // at their offsets.  states: evaluate the walls' states once a step
@@ -374,6 +378,7 @@ bool res_states_pass(const WallArgs<C> *wall)
 {
     return (wall[WEST].needs_data || wall[EAST].needs_data) && (wall[SOUTH].needs_data || wall[NORTH].needs_data);
 }
+int resident_plan_capacity(int ex, int threads, size_t smem, bool states);
 cudaError_t launch_resident_plan(const BatchDesc<float, float> *descs, const ResPlanTile *tiles, int ntiles, int ex,
                                  int threads, size_t smem, bool states, int parity, int nsteps, void *xchg,
                                  unsigned tag, unsigned *err, unsigned long long timeout_ns, cudaStream_t stream);

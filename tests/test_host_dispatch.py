@@ -35,15 +35,15 @@ FAKE = r"""
 using namespace lbm13;
 
 // what the stand-in does: the n-th next memset, allocation or resident launch fails;
-// attributes; the capture status of every stream but those the library makes
+// attributes; whether the lattice's stream, or another one of the process, is captured
 extern "C" {
 int fake_fail_memset = 0, fake_fail_malloc = 0, fake_fail_resident = 0, fake_cooperative = 1, fake_capturing = 0,
-    fake_blocks_per_sm = 1;
+    fake_blocks_per_sm = 1, fake_other_capture = 0;
 }
 static std::string g_log;
 static std::map<void *, size_t> g_mem;
 static std::set<void *> g_own;
-static bool g_capture = false;
+static bool g_capture = false, g_relaxed = false;
 extern "C" const char *fake_log() { return g_log.c_str(); }
 extern "C" void fake_clear() { g_log.clear(); }
 extern "C" int fake_allocations() { return int(g_mem.size()); }
@@ -54,6 +54,7 @@ extern "C" {
 cudaError_t cudaMalloc(void **p, size_t n)
 {
     if (hit(fake_fail_malloc)) return cudaErrorMemoryAllocation;
+    if (fake_other_capture && !g_relaxed) return cudaErrorStreamCaptureUnsupported;
     *p = std::malloc(n);
     std::memset(*p, 0xa5, n);  // as memory comes
     g_mem[*p] = n;
@@ -107,7 +108,13 @@ cudaError_t cudaGraphInstantiate(cudaGraphExec_t *x, cudaGraph_t, unsigned long 
 cudaError_t cudaGraphDestroy(cudaGraph_t g) { std::free(g); return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t x) { std::free(x); return cudaSuccess; }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { g_log += "g "; return cudaSuccess; }
-cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *) { return cudaSuccess; }
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *m)
+{
+    const cudaStreamCaptureMode old = g_relaxed ? cudaStreamCaptureModeRelaxed : cudaStreamCaptureModeGlobal;
+    g_relaxed = *m == cudaStreamCaptureModeRelaxed;
+    *m = old;
+    return cudaSuccess;
+}
 cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **p, unsigned, unsigned long long, cudaDriverEntryPointQueryResult *q)
 {
     *p = reinterpret_cast<void *>(&fake_encode);
@@ -180,7 +187,11 @@ cudaError_t launch_resident(const StepArgs<T, C> &a, bool, int n, const ResShape
 }
 cudaError_t launch_resident_plan(const BatchDesc<float, float> *, const ResPlanTile *, int, int, int, size_t, bool, int, int n,
                                  void *, unsigned, unsigned *, unsigned long long, cudaStream_t) { return resident("P", n); }
+template <typename T, typename C>
+int resident_capacity(const ResShape &, bool, const WallArgs<C> *) { return 152 * fake_blocks_per_sm; }
+int resident_plan_capacity(int, int, size_t, bool) { return 152 * fake_blocks_per_sm; }
 #define BOTH(T) \
+    template int resident_capacity<T, T>(const ResShape &, bool, const WallArgs<T> *); \
     template cudaError_t launch_multi<T, T>(const StepArgs<T, T> &, const StepArgs<T, T> &, bool, int, int, const GridSync &, cudaStream_t); \
     template cudaError_t launch_step<T, T>(const StepArgs<T, T> &, bool, cudaStream_t); \
     template cudaError_t launch_batch<T, T>(const BatchDesc<T, T> *, const int2 *, int, int, int, int, int, int, cudaStream_t); \
@@ -212,6 +223,7 @@ def lib(tmp_path_factory):
     L.fake_log.restype = C.c_char_p
     L.lbm13_last_error.restype = C.c_char_p
     L.lbm13_plan_last_error.restype = C.c_char_p
+    L.lbm13_time.restype = C.c_int64
     return L
 
 
@@ -249,7 +261,7 @@ def _set(L, **kw):
 @pytest.fixture(autouse=True)
 def _defaults(lib):
     yield
-    _set(lib, fail_memset=0, fail_malloc=0, fail_resident=0, cooperative=1, capturing=0, blocks_per_sm=1)
+    _set(lib, fail_memset=0, fail_malloc=0, fail_resident=0, cooperative=1, capturing=0, blocks_per_sm=1, other_capture=0)
 
 
 def _cavity(**kw):
@@ -289,4 +301,76 @@ def test_a_work_space_that_could_not_be_cleared_is_made_again(lib, call):
     assert f() == 0
     assert not any("NOT-CLEARED" in x for x in a.log()), a.log()
     a.close()
+    assert lib.fake_allocations() == 0
+
+
+def test_launches_of_a_run(lib):
+    """By mode, length and size; asking for their number makes and allocates nothing."""
+    n = C.c_int64()
+    for nx, ny, prec, mode, steps, want in [
+            (64, 64, FP32, AUTO, 64, ["R64"]), (64, 64, FP32, AUTO, 31, ["s"] * 31), (64, 64, FP32, OFF, 64, ["g", "g"]),
+            (64, 64, FP32, ON, 2, ["R2"]), (900, 900, FP32, AUTO, 64, ["g", "g"]), (900, 900, FP32, ON, 64, ["M64"]),
+            (64, 64, FP64, AUTO, 32, ["R32"]), (64, 64, FP64, ON, 1, ["s"])]:
+        a = Lat(lib, nx, ny, prec, _cavity(), mode)
+        held = lib.fake_allocations()
+        assert lib.lbm13_step_launches(a.h, C.c_int64(steps), C.byref(n)) == 0
+        assert lib.fake_allocations() == held and a.log() == []
+        st, log = a.step(steps)
+        assert st == 0 and log == want, (nx, prec, mode, steps, log)
+        per_graph = {"g": 32}
+        assert n.value == sum(per_graph.get(x, 1) for x in log)
+        a.close()
+
+
+@pytest.mark.parametrize("mode", [AUTO, ON])
+def test_a_refused_launch_from_shared_memory_leaves_the_steps_to_others(lib, mode):
+    a = Lat(lib, 64, 64, FP32, _cavity(), mode)
+    _set(lib, fail_resident=1)
+    st, log = a.step(70)
+    assert st == 0 and log == (["M70"] if mode == ON else ["g", "g"] + ["s"] * 6), log
+    assert lib.lbm13_time(a.h) == 70
+    a.close()
+    b = Lat(lib, 64, 64, FP32, _cavity(), mode)
+    _set(lib, fail_resident=2)  # the second of three launches
+    st, log = b.step(1024 + 1024 + 64)
+    assert st == 0 and log[0] == "R1024" and not any(x.startswith("R") for x in log[1:])
+    assert lib.lbm13_time(b.h) == 2112
+    b.close()
+
+
+def test_no_launch_from_shared_memory_where_its_blocks_do_not_fit_at_once(lib):
+    _set(lib, blocks_per_sm=0)
+    a = Lat(lib, 64, 64, FP32, _cavity())
+    assert a.step(64) == (0, ["g", "g"])
+    a.close()
+
+
+def test_a_run_allocates_beside_a_capture_elsewhere(lib):
+    a = Lat(lib, 64, 64, FP32, _cavity())
+    _set(lib, other_capture=1)
+    assert a.step(64) == (0, ["R64"])
+    _set(lib, other_capture=0, capturing=1)  # its own stream is captured: the launches that are recorded
+    assert a.step(33) == (0, ["g", "s"])
+    a.close()
+
+
+def _plan(lib, lats):
+    arr = (C.c_void_p * len(lats))(*[a.h for a in lats])
+    p = C.c_void_p()
+    assert lib.lbm13_plan_create(arr, len(lats), None, None, C.byref(p)) == 0
+    return p
+
+
+def test_a_refused_plan_launch_leaves_the_steps_to_others(lib):
+    lats = [Lat(lib, 64, 64, FP32, _cavity()) for _ in range(3)]
+    p = _plan(lib, lats)
+    lib.fake_clear()
+    assert lib.lbm13_plan_step(p, C.c_int64(64)) == 0 and lats[0].log() == ["P64"]
+    _set(lib, fail_resident=1)
+    lib.fake_clear()
+    assert lib.lbm13_plan_step(p, C.c_int64(65)) == 0 and lats[0].log() == ["g", "g", "b"]
+    assert [lib.lbm13_time(a.h) for a in lats] == [129] * 3
+    lib.lbm13_plan_destroy(p)
+    for a in lats:
+        a.close()
     assert lib.fake_allocations() == 0
