@@ -256,9 +256,11 @@ int lbm13_info(lbm13_t h, int64_t out[8]);
  * 600^2 nodes in FP32-deviation storage, 350^2 in FP64) stays in it, one tile a
  * block, and neighbouring blocks exchange the nodes around their tiles through
  * L2; others step in global memory with grid barriers.
- * AUTO (default): from shared memory where the lattice fits, for n >= 32 (on
- * GB300 two to six times faster than per-step launches there), otherwise
- * per-step launches; OFF: per-step launches; ON: from shared memory where the
+ * AUTO (default): from shared memory for n >= 32 where the lattice fits, in FP64
+ * up to 131,072 nodes or with temperature or moving walls on both axes, otherwise
+ * per-step launches.  On GB300 that is 1.06 to 2.6 times as fast as per-step
+ * launches in FP32, and 0.92 (channels of 131,072 nodes) to 2.0 times in FP64;
+ * OFF: per-step launches; ON: from shared memory where the
  * lattice fits, else with grid barriers whenever a cooperative launch is
  * possible.  Slabs (LBM13_HALO sides) and streams under capture take per-step
  * launches.  The exchange buffer (160 bytes per node in FP32-deviation storage,

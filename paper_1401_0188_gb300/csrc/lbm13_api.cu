@@ -378,9 +378,26 @@ int ensure_sync_mem(lbm13_t h)
     return dev_zeroed(h, h->sync_mem, kSyncBytes, 0, kSyncBytes, h->stream, "the step error word");
 }
 
+// FP64 gains less from shared memory, its step being bound by integer instructions in
+// either case: up to 2^17 nodes, or any number that fits where walls of both axes need
+// data (edge links cost single launches more there).  Microseconds a step, single
+// launches and from shared memory: periodic 128^2 5.8 and 2.9, 256^2 7.6 and 6.2, 360^2
+// 11.6 and 10.8, 400^2 12.5 and 13.5; cavity 128^2 7.1 and 5.4, 256^2 10.4 and 9.9, 360^2
+// 14.8 and 14.3, 400^2 16.2 and 18.0, 1024 x 128 13.4 and 14.2; channels (y walls only)
+// 224^2 7.8 and 8.4, 1024 x 64 8.7 and 8.4, 1024 x 128 11.6 and 12.5; box 256^2 17.6 and
+// 12.4, 440^2 24.7 and 22.3.  FP32: 1.06 to 2.6 times faster wherever a split fits.
+constexpr long long kResMaxNodes64 = 1LL << 17;
+
+bool resident_pays(lbm13_t h)
+{
+    return h->precision != LBM13_FP64 || h->persistent == LBM13_PERSISTENT_ON ||
+           (long long)h->nx * h->ny <= kResMaxNodes64 || res_states_pass(h->wd);
+}
+
 // Whether lbm13_step takes n steps from shared memory (resident_kernel): where a
-// split of the lattice fits the SMs, for kResMinSteps steps or more (a launch
-// loads and stores the whole state once), or for any n >= 2 in persistent mode.
+// split of the lattice fits the SMs and is the faster way (resident_pays), for
+// kResMinSteps steps or more (a launch loads and stores the whole state once), or for
+// any n >= 2 in persistent mode.
 // A slab's halo rows change between steps, and a stream that is being captured
 // keeps the launches it would have recorded before.
 constexpr long long kResMinSteps = 32;
@@ -390,6 +407,7 @@ bool wants_resident(lbm13_t h, long long n)
     if (h->persistent == LBM13_PERSISTENT_OFF || n < (h->persistent == LBM13_PERSISTENT_ON ? 2 : kResMinSteps) ||
         h->b.south.kind == HALO || h->b.north.kind == HALO)
         return false;
+    if (!resident_pays(h)) return false;
     if (h->res.ex < 0) {
         int dev = 0, coop = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||

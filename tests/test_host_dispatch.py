@@ -322,6 +322,21 @@ def test_launches_of_a_run(lib):
         a.close()
 
 
+def test_large_fp64_lattices_step_launch_by_launch(lib):
+    """Where shared memory holds them but single launches are faster."""
+    M, BB = W.WALL_MIXED, W.WALL_BB
+    T0 = rest_temperature(pstar(0.05, 0.71))
+    box = W.boundary(west=W.wall(M, 0.0, T0), east=W.wall(BB), south=W.wall(M, 0.01, T0), north=W.wall(BB))
+    for nx, ny, prec, bnd, mode, want in [
+            (362, 362, FP64, _cavity(), AUTO, "R"), (363, 362, FP64, _cavity(), AUTO, "g"), (500, 500, FP64, None, AUTO, "g"),
+            (1024, 128, FP64, None, AUTO, "R"), (440, 440, FP64, box, AUTO, "R"), (440, 440, FP64, _cavity(), ON, "R"),
+            (600, 600, FP32, _cavity(), AUTO, "R")]:
+        a = Lat(lib, nx, ny, prec, bnd, mode)
+        st, log = a.step(64)
+        assert st == 0 and log[0][0] == want, (nx, ny, prec, mode, log)
+        a.close()
+
+
 @pytest.mark.parametrize("mode", [AUTO, ON])
 def test_a_refused_launch_from_shared_memory_leaves_the_steps_to_others(lib, mode):
     a = Lat(lib, 64, 64, FP32, _cavity(), mode)
