@@ -253,7 +253,7 @@ int lbm13_info(lbm13_t h, int64_t out[8]);
  * graphs in runs of 32), or launches that advance the lattice by up to 1024
  * steps in one cooperative launch (results are bit-identical).  There are two
  * of those: a lattice whose populations fit the SMs' shared memory (up to about
- * 600^2 nodes in FP32-deviation storage, 350^2 in FP64) stays in it, one tile a
+ * 660^2 nodes in FP32-deviation storage, 440^2 in FP64) stays in it, one tile a
  * block, and neighbouring blocks exchange the nodes around their tiles through
  * L2; others step in global memory with grid barriers.
  * AUTO (default): from shared memory for n >= 32 where the lattice fits, in FP64
@@ -307,6 +307,16 @@ int lbm13_step_launches(lbm13_t h, int64_t n, int64_t *launches);
  * word was set (it is cleared again); the state and the step counter stay
  * as they were.  LBM13_EINVAL for a lattice that does not take paired steps. */
 int lbm13_pair_check(lbm13_t h, double timeout_s, int withhold, int *timed_out);
+
+/* Self-check of the bounded wait of stepping from shared memory: one launch of
+ * three steps from the current state with its waits limited to timeout_s (1e-3 ..
+ * 2 s) and, when withhold != 0, without the last tile, so that the waits for its
+ * nodes run out and the blocks report and leave.  *timed_out = 1 when the error word
+ * was set; it is cleared again, or with withhold = 2 left for the next synchronising
+ * call to report (LBM13_ETIMEOUT).  The state and the step counter stay as they
+ * were.  LBM13_EINVAL for a lattice that does not step from shared memory in two
+ * tiles or more. */
+int lbm13_resident_check(lbm13_t h, double timeout_s, int withhold, int *timed_out);
 
 /* Self-check of the grid barrier's bounded wait on the current device: a
  * cooperative launch of `blocks` blocks runs 4 barriers that wait for
@@ -478,6 +488,11 @@ int lbm13_plan_set_config(lbm13_plan_t p, int R, int BY, int ctas_per_sm, int or
  * in such a launch either).  *timed_out = 1 when the error word was set (it is cleared
  * again).  The plan does not advance: the lattices keep their states. */
 int lbm13_plan_tma_check(lbm13_plan_t p, double timeout_s, int withhold, int *timed_out);
+
+/* The same self-check as lbm13_resident_check for a plan that steps from shared
+ * memory (else LBM13_EINVAL); with withhold = 2 lbm13_plan_residual reports the
+ * timeout. */
+int lbm13_plan_resident_check(lbm13_plan_t p, double timeout_s, int withhold, int *timed_out);
 
 /* out: R, BY, ctas_per_sm, order, tiles, grid, total nodes, candidates tried
  * by the last tune, groups. */

@@ -946,6 +946,37 @@ int lbm13_pair_check(lbm13_t h, double timeout_s, int withhold, int *timed_out)
     return LBM13_OK;
 }
 
+int lbm13_resident_check(lbm13_t h, double timeout_s, int withhold, int *timed_out)
+{
+    if (!h || !timed_out || !(timeout_s >= 1e-3 && timeout_s <= 2.0))
+        return fail(h, LBM13_EINVAL, "NULL argument or timeout_s outside [1e-3, 2]");
+    DeviceGuard g(h->device);
+    if (!use_resident(h, kResMinSteps) || h->res.gx * h->res.gy < 2)
+        return fail(h, LBM13_EINVAL, "the lattice does not step from shared memory in two tiles or more");
+    SYNC_CHECK(h);
+    // an odd number of steps: what is written is not the state's buffer
+    const int n = 3, x = res_exchanges(h->res.K, n);
+    if (h->res_tag > 0xffffffffu - unsigned(x)) {
+        CK(h, cudaMemsetAsync(h->res_xchg, 0, res_exchange_bytes(h->nx, h->ny, int(h->elem)), h->stream));
+        h->res_tag = 0;
+    }
+    const unsigned long long ns = (unsigned long long)(timeout_s * 1e9);
+    const int absent = withhold ? 1 : 0;
+    cudaError_t e = h->precision == LBM13_FP64
+                        ? launch_resident<double, double>(step_args<double, double>(h, h->cur, h->kd, h->wd), h->force, n,
+                                                          h->res, h->res_xchg, h->res_tag, step_err(h), ns, h->stream, absent)
+                        : launch_resident<float, float>(step_args<float, float>(h, h->cur, h->kf, h->wf), h->force, n,
+                                                        h->res, h->res_xchg, h->res_tag, step_err(h), ns, h->stream, absent);
+    h->res_tag += unsigned(x);
+    unsigned word = 0;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) e = cudaMemcpy(&word, step_err(h), sizeof word, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess && withhold != 2) e = cudaMemset(h->sync_mem, 0, kSyncBytes);
+    if (e != cudaSuccess) return cuda_fail(h, e, "resident step check");
+    *timed_out = word != 0u;
+    return LBM13_OK;
+}
+
 int lbm13_set_persistent(lbm13_t h, int mode)
 {
     if (!h) return fail(nullptr, LBM13_EINVAL, "NULL handle");
@@ -2056,6 +2087,39 @@ int lbm13_plan_tma_check(lbm13_plan_t p, double timeout_s, int withhold, int *ti
     if (e == cudaSuccess) e = cudaMemcpy(&word, p->tma_err, sizeof word, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemset(p->tma_err, 0, sizeof word);
     if (e != cudaSuccess) return pfail(p, LBM13_ECUDA, std::string("staged tile check: ") + cudaGetErrorString(e));
+    *timed_out = word != 0u;
+    return LBM13_OK;
+}
+
+int lbm13_plan_resident_check(lbm13_plan_t p, double timeout_s, int withhold, int *timed_out)
+{
+    if (!p || !timed_out || !(timeout_s >= 1e-3 && timeout_s <= 2.0))
+        return pfail(p, LBM13_EINVAL, "NULL argument or timeout_s outside [1e-3, 2]");
+    DeviceGuard g(p->device);
+    int rc = plan_sync_parity(p);
+    bool use = false;
+    if (rc == LBM13_OK) rc = plan_use_resident(p, kResMinSteps, use);
+    if (rc != LBM13_OK) return rc;
+    if (!use || p->res_ntiles < 2)
+        return pfail(p, LBM13_EINVAL, "the plan does not step from shared memory in two tiles or more");
+    const int n = 3;  // odd: what is written is not the states' buffers
+    const unsigned x = unsigned(res_exchanges(p->res_min_k, n));
+    cudaError_t e = cudaSuccess;
+    if (p->res_tag > 0xffffffffu - x) {
+        e = cudaMemsetAsync(p->res_xchg, 0, p->res_xchg_bytes, p->stream);
+        p->res_tag = 0;
+    }
+    if (e == cudaSuccess)
+        e = launch_resident_plan(static_cast<const BatchDesc<float, float> *>(p->desc),
+                                 static_cast<const ResPlanTile *>(p->res_tiles), p->res_ntiles - (withhold ? 1 : 0),
+                                 p->res_ex, p->res_threads, p->res_smem_bytes, p->res_states, p->parity, n, p->res_xchg,
+                                 p->res_tag, p->tma_err, (unsigned long long)(timeout_s * 1e9), p->stream);
+    p->res_tag += x;
+    unsigned word = 0;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
+    if (e == cudaSuccess) e = cudaMemcpy(&word, p->tma_err, sizeof word, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess && withhold != 2) e = cudaMemset(p->tma_err, 0, sizeof word);
+    if (e != cudaSuccess) return pfail(p, LBM13_ECUDA, std::string("resident plan check: ") + cudaGetErrorString(e));
     *timed_out = word != 0u;
     return LBM13_OK;
 }

@@ -443,7 +443,7 @@ int res_capacity(const void *fn, int threads, size_t smem)
 
 template <typename T, typename C>
 cudaError_t launch_resident(const StepArgs<T, C> &a, bool force, int nsteps, const ResShape &s, void *xchg,
-                            unsigned tag, unsigned *err, unsigned long long timeout_ns, cudaStream_t stream)
+                            unsigned tag, unsigned *err, unsigned long long timeout_ns, cudaStream_t stream, int absent)
 {
     const void *fn = nullptr;
     const cudaError_t e = resident_ready<T, C>(s, force, res_states_pass(a.wall), fn);
@@ -453,7 +453,7 @@ cudaError_t launch_resident(const StepArgs<T, C> &a, bool force, int nsteps, con
     ResShape ps = s;
     unsigned char *px = static_cast<unsigned char *>(xchg);
     void *args[] = {&pa, &ps, &nsteps, &px, &tag, &err, &timeout_ns};
-    return cudaLaunchCooperativeKernel(fn, dim3(s.gx * s.gy), dim3(s.threads), args,
+    return cudaLaunchCooperativeKernel(fn, dim3(s.gx * s.gy - absent), dim3(s.threads), args,
                                        res_smem(s, int(sizeof(T))), stream);
 }
 
@@ -492,8 +492,8 @@ cudaError_t launch_resident_plan(const BatchDesc<float, float> *descs, const Res
 template int resident_capacity<double, double>(const ResShape &, bool, const WallArgs<double> *);
 template int resident_capacity<float, float>(const ResShape &, bool, const WallArgs<float> *);
 template cudaError_t launch_resident<double, double>(const StepArgs<double, double> &, bool, int, const ResShape &,
-                                                     void *, unsigned, unsigned *, unsigned long long, cudaStream_t);
+                                                     void *, unsigned, unsigned *, unsigned long long, cudaStream_t, int);
 template cudaError_t launch_resident<float, float>(const StepArgs<float, float> &, bool, int, const ResShape &, void *,
-                                                   unsigned, unsigned *, unsigned long long, cudaStream_t);
+                                                   unsigned, unsigned *, unsigned long long, cudaStream_t, int);
 
 } // namespace lbm13

@@ -343,7 +343,8 @@ inline double res_plan_shapes(const std::vector<ResLattice> &lats, int elem, int
 // first exchange of every block that reads nodes of that tile.  xchg: res_exchange_bytes bytes, zeroed once; the launch's exchanges
 // are numbered tag + 1, tag + 2, ... (res_exchanges of them), which must not have
 // been used before.  A wait that runs out (timeout_ns) sets *err, and the block
-// leaves without writing.
+// leaves without writing.  absent: that many tiles, the last ones, are not launched,
+// so that the waits for them run out (a self-check).
 // Steps between two exchanges of a launch: at least one exchange for two steps or more.
 LBM13_HD constexpr int res_between(int K, int nsteps) { return nsteps > K ? K : (nsteps + 1) / 2; }
 LBM13_HD constexpr int res_exchanges(int K, int nsteps)
@@ -352,7 +353,8 @@ LBM13_HD constexpr int res_exchanges(int K, int nsteps)
 }
 template <typename T, typename C>
 cudaError_t launch_resident(const StepArgs<T, C> &a, bool force, int nsteps, const ResShape &s, void *xchg,
-                            unsigned tag, unsigned *err, unsigned long long timeout_ns, cudaStream_t stream);
+                            unsigned tag, unsigned *err, unsigned long long timeout_ns, cudaStream_t stream,
+                            int absent = 0);
 
 // Blocks of such a launch that the SMs hold at once (0 where it cannot be launched).
 template <typename T, typename C>

@@ -40,9 +40,9 @@ EXPORTS = ("lbm13_version", "lbm13_status_string", "lbm13_derive", "lbm13_create
            "lbm13_plan_last_error", "lbm13_plan_step", "lbm13_plan_tune", "lbm13_plan_set_config",
            "lbm13_plan_config", "lbm13_plan_residual", "lbm13_totals_noalloc", "lbm13_project",
            "lbm13_set_persistent", "lbm13_barrier_check", "lbm13_linear_growth", "lbm13_debug_violations",
-           "lbm13_plan_tma_check", "lbm13_fp64_fma_rate", "lbm13_plan_add", "lbm13_plan_remove",
+           "lbm13_plan_tma_check", "lbm13_plan_resident_check", "lbm13_fp64_fma_rate", "lbm13_plan_add", "lbm13_plan_remove",
            "lbm13_halo_bytes", "lbm13_halo_pack", "lbm13_halo_unpack", "lbm13_linear_growth_batch",
-           "lbm13_set_pair_steps", "lbm13_step_launches", "lbm13_pair_check")
+           "lbm13_set_pair_steps", "lbm13_step_launches", "lbm13_pair_check", "lbm13_resident_check")
 
 
 class Lbm13Error(RuntimeError):
@@ -118,11 +118,13 @@ def lib():
         "lbm13_set_pair_steps": (C.c_int, [vp, C.c_int]),
         "lbm13_step_launches": (C.c_int, [vp, i64, C.POINTER(i64)]),
         "lbm13_pair_check": (C.c_int, [vp, C.c_double, C.c_int, C.POINTER(C.c_int)]),
+        "lbm13_resident_check": (C.c_int, [vp, C.c_double, C.c_int, C.POINTER(C.c_int)]),
         "lbm13_linear_growth": (C.c_int, [C.POINTER(Params), C.c_double, C.c_double, C.c_int, C.POINTER(C.c_double)]),
         "lbm13_barrier_check": (C.c_int, [C.c_int, C.c_int, C.c_double, C.POINTER(C.c_int)]),
         "lbm13_linear_growth_batch": (C.c_int, [C.POINTER(Params), dp, dp, C.c_int, C.c_int, dp, vp]),
         "lbm13_debug_violations": (C.c_int, [vp, C.POINTER(C.c_ulonglong)]),
         "lbm13_plan_tma_check": (C.c_int, [vp, C.c_double, C.c_int, C.POINTER(C.c_int)]),
+        "lbm13_plan_resident_check": (C.c_int, [vp, C.c_double, C.c_int, C.POINTER(C.c_int)]),
         "lbm13_time": (i64, [vp]),
         "lbm13_synchronize": (C.c_int, [vp]),
         "lbm13_totals_noalloc": (C.c_int, [vp, vp]),
@@ -442,6 +444,13 @@ class Lattice:
         _check(lib().lbm13_pair_check(self._h, float(timeout_s), int(bool(withhold)), C.byref(out)), self._h)
         return bool(out.value)
 
+    def resident_check(self, timeout_s, withhold=1):
+        """Self-check of the bounded wait of stepping from shared memory; True when it
+        ran out (withhold=2: the next synchronising call reports the timeout)."""
+        out = C.c_int()
+        _check(lib().lbm13_resident_check(self._h, float(timeout_s), int(withhold), C.byref(out)), self._h)
+        return bool(out.value)
+
     def project(self, kx, ky=0):
         """Fourier aggregates (Sec. 6): [field][harmonic][cos, sin] for the
         fields (rho - 1, ux, uy, T - T0, E - E0, p - T0), harmonics k and 2k of
@@ -534,6 +543,13 @@ class Plan:
         ran out (expected exactly when the copies are withheld)."""
         out = C.c_int(0)
         _pcheck(lib().lbm13_plan_tma_check(self._h, float(timeout_s), 1 if withhold else 0, C.byref(out)), self._h)
+        return bool(out.value)
+
+    def resident_check(self, timeout_s, withhold=1):
+        """Self-check of the bounded wait of stepping from shared memory; True when it
+        ran out (withhold=2: residual() reports the timeout)."""
+        out = C.c_int(0)
+        _pcheck(lib().lbm13_plan_resident_check(self._h, float(timeout_s), int(withhold), C.byref(out)), self._h)
         return bool(out.value)
 
     def config(self):

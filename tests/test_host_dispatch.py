@@ -177,7 +177,7 @@ cudaError_t launch_project(const ReadArgs<T> &, int, int, double *, int, unsigne
 }
 template <typename T, typename C>
 cudaError_t launch_resident(const StepArgs<T, C> &a, bool, int n, const ResShape &, void *xchg, unsigned, unsigned *err,
-                            unsigned long long, cudaStream_t)
+                            unsigned long long, cudaStream_t, int)
 {
     const unsigned *w = static_cast<const unsigned *>(xchg);
     for (size_t i = 3; i < res_exchange_bytes(a.nx, a.ny, sizeof(T)) / 4; i += 4)
@@ -201,7 +201,7 @@ int resident_plan_capacity(int, int, size_t, bool) { return 152 * fake_blocks_pe
     template cudaError_t launch_reduce<T>(const ReduceJob<T> &, cudaStream_t); \
     template cudaError_t launch_reduce_batch<T>(const ReduceJob<T> *, int, int, cudaStream_t); \
     template cudaError_t launch_project<T>(const ReadArgs<T> &, int, int, double *, int, unsigned *, double *, cudaStream_t); \
-    template cudaError_t launch_resident<T, T>(const StepArgs<T, T> &, bool, int, const ResShape &, void *, unsigned, unsigned *, unsigned long long, cudaStream_t);
+    template cudaError_t launch_resident<T, T>(const StepArgs<T, T> &, bool, int, const ResShape &, void *, unsigned, unsigned *, unsigned long long, cudaStream_t, int);
 BOTH(float)
 BOTH(double)
 }
