@@ -58,6 +58,20 @@ struct SharedSrc {
     }
 };
 
+// Debug builds: a population of the shared rows [0, n) reached by pointer; an access
+// outside is counted and goes to the first one instead.
+template <typename T, typename C>
+__device__ __forceinline__ T *chk_shared(const StepArgs<T, C> &a, T *rows, size_t n, T *p)
+{
+#ifdef LBM13_DEBUG
+    if (p < rows || p >= rows + n) {
+        atomicAdd(a.bad, 1ull);
+        return rows;
+    }
+#endif
+    return p;
+}
+
 // One 16-byte unit of the exchange buffer, written and read as one access.
 struct Unit {
     unsigned long long lo, hi;
@@ -131,7 +145,8 @@ __device__ __forceinline__ void resident_tile(const StepArgs<T, C> &a, bool forc
     constexpr int kFar = 1 << 24;  // where a periodic axis' node 0 lies in sa's coordinates
     constexpr int kUnits = res_units(sizeof(T));
     T *const sm = reinterpret_cast<T *>(res_mem);
-    T *const links = sm + size_t(s.rows) * Q * EX;  // [13][span]
+    const size_t held = size_t(s.rows) * Q * EX;
+    T *const links = sm + held;  // [13][span]
     const int along = res_along(s);
     T *const states = links + size_t(s.edges) * Q;  // [4][along] pairs: the walls' density and energy
     unsigned *const found = reinterpret_cast<unsigned *>(states + size_t(8) * along);  // [13][span]
@@ -157,7 +172,7 @@ __device__ __forceinline__ void resident_tile(const StepArgs<T, C> &a, bool forc
         for (int j = 0; j < Q; ++j)
             v[j] = __ldcg(chk(a, a.fin, a.fin + (long long)y * a.pitch + x + (long long)j * a.plane));
 #pragma unroll
-        for (int j = 0; j < Q; ++j) p[j * EX] = v[j];
+        for (int j = 0; j < Q; ++j) *chk_shared(a, sm, held, p + j * EX) = v[j];
     }
     __syncthreads();
     // the edge nodes, numbered as in the largest region: column and row in the
@@ -228,7 +243,7 @@ __device__ __forceinline__ void resident_tile(const StepArgs<T, C> &a, bool forc
                 for (int j = 0; j < Q; ++j) {
                     T v;
                     res_value(w, v, j);
-                    p[j * EX] = v;
+                    *chk_shared(a, sm, held, p + j * EX) = v;
                 }
             }
             if (__syncthreads_or(!ok)) return;
@@ -307,7 +322,7 @@ __device__ __forceinline__ void resident_tile(const StepArgs<T, C> &a, bool forc
                 C f[Q];
                 if (valid && !edge) {
 #pragma unroll
-                    for (int j = 0; j < Q; ++j) f[j] = C(p[(j - Q * cvy(j)) * EX - cvx(j)]);
+                    for (int j = 0; j < Q; ++j) f[j] = C(*chk_shared(a, sm, held, p + ((j - Q * cvy(j)) * EX - cvx(j))));
                 }
                 __syncthreads();  // every read of the chunk before its writes
                 if (valid) {
@@ -321,7 +336,7 @@ __device__ __forceinline__ void resident_tile(const StepArgs<T, C> &a, bool forc
                     else
                         collide<false>(f, a.k);
 #pragma unroll
-                    for (int j = 0; j < Q; ++j) p[j * EX + shift] = T(f[j]);
+                    for (int j = 0; j < Q; ++j) *chk_shared(a, sm, held, p + (j * EX + shift)) = T(f[j]);
                     if (k == 0 && last) {
                         store(a, x, y, f);
                     } else if (k == 0 && (x < t.x0 + 2 * K || x >= t.x1 - 2 * K || y < t.y0 + 2 * K ||

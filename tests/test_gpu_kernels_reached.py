@@ -1,4 +1,13 @@
-"""The bounded wait of stepping from shared memory, made to run out."""
+"""Kernels that the default modes reach at some sizes only, each on lattices that do
+reach it: grid-barrier launches of lattices that shared memory does not hold, the
+ring-staged strips through 32-step graphs, the walled per-step kernels and the shared
+rows in the bounds-checked build, and the bounded wait of stepping from shared memory
+made to run out."""
+import json
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -6,6 +15,7 @@ from paper_1401_0188_gb300 import pstar as product_pstar
 from paper_1401_0188_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -31,6 +41,42 @@ def _lattice(L, nx, ny, kind, precision, mode, stream=None):
     g.set_persistent(mode)
     g.set_state(*W.random_fields(nx, ny, T0, seed=nx + ny, du=0.01, drho=0.005, dT=0.003))
     return g
+
+
+@pytest.mark.parametrize("kind", ["periodic", "cavity", "cavity_zero_flux", "couette", "box"])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_grid_barrier_launches_of_lattices_that_shared_memory_does_not_hold(L, kind, precision):
+    nx, ny = (901, 803) if precision else (571, 502)  # more populations than the SMs hold
+    a = _lattice(L, nx, ny, kind, precision, L.PERSISTENT_ON)
+    b = _lattice(L, nx, ny, kind, precision, L.PERSISTENT_OFF)
+    held = a.info()["device_bytes"]
+    assert a.step_launches(40) == 1
+    for n in (2, 33, 1031 if kind == "cavity" else 7):  # the longest takes two launches
+        a.step(n)
+        b.step(n)
+        assert a.save() == b.save(), n
+    # the grid of the barrier kernel, and no exchange buffer: nothing was stepped from
+    # shared memory
+    assert a.info()["persistent_grid"] > 0 and a.info()["device_bytes"] - held < 4096
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("BY", [8, 4])
+def test_ring_strips_through_graphs_on_lattices_that_step_launch_by_launch(L, BY):
+    sizes = [(300, 260, "cavity"), (257, 131, "periodic"), (128, 640, "couette"), (64, 64, "box")]
+    a = [_lattice(L, nx, ny, k, 1, L.PERSISTENT_OFF) for nx, ny, k in sizes]
+    b = [_lattice(L, nx, ny, k, 1, L.PERSISTENT_OFF) for nx, ny, k in sizes]
+    plan = L.Plan(a)
+    for groups in (3, 16):
+        plan.set_config(0, BY, 0, 2, groups)
+        plan.step(35)  # one 32-step graph and three launches
+        for x, y in zip(a, b):
+            y.step(35)
+            assert x.save() == y.save()
+    with pytest.raises(L.Lbm13Error):
+        plan.resident_check(0.02)  # the plan does not step from shared memory
+    plan.close()
 
 
 @pytest.mark.parametrize("kind", ["periodic", "cavity", "box"])
@@ -86,3 +132,48 @@ def test_the_wait_between_tiles_of_a_plan_is_bounded(L):
         assert x.save() == y.save()
     plan.close()
 
+
+SCRIPT = r"""
+import json
+import torch
+from paper_1401_0188_gb300 import lbm13, params as P, workloads as W
+
+p = P.pstar(0.05, 0.71)
+T0 = P.rest_temperature(p)
+M, B = W.WALL_MIXED, W.WALL_BB
+box = W.boundary(west=W.wall(M, -0.01, T0 + 0.005), east=W.wall(M, 0.015, T0 - 0.005), south=W.wall(M, 0.02, T0),
+                 north=W.wall(M, -0.01, T0))
+cases = [(48, 40, W.cavity(T0, 0.01, 2e-4)), (37, 30, W.couette(T0, 0.05, 0.01)), (34, 29, box), (4, 4, box),
+         (100, 70, W.cavity(T0, 0.01, 1e-4, wall_density=1)), (40, 24, W.heated_slab(T0, 1e-5, 0.02)), (131, 97, W.boundary(gx=1e-5))]
+launches, lats = {"step": 0, "resident": 0, "barrier": 0}, []
+
+
+def run(nx, ny, bnd, prec, mode, n, kind):
+    g = lbm13.Lattice(nx, ny, p, bnd, precision=prec)
+    g.set_persistent(mode)
+    g.set_state(*W.random_fields(nx, ny, T0, 7, du=0.01, drho=0.005, dT=0.003))
+    launches[kind] += g.step_launches(n) == (n if kind == "step" else 1)
+    g.step(n)
+    g.step(3)
+    lats.append(g)
+
+
+for prec in (lbm13.FP64, lbm13.FP32_DEVIATION):
+    for nx, ny, bnd in cases:
+        run(nx, ny, bnd, prec, lbm13.PERSISTENT_OFF, 37, "step")
+        run(nx, ny, bnd, prec, lbm13.PERSISTENT_AUTO, 37, "resident")
+    for bnd in (box, W.boundary(), W.cavity(T0, 0.01, 1e-4)):
+        run(901, 803, bnd, prec, lbm13.PERSISTENT_ON, 5, "barrier")
+torch.cuda.synchronize()
+print(json.dumps(dict(launches, violations=sum(g.debug_violations() for g in lats))))
+"""
+
+
+def test_every_way_of_stepping_stays_inside_the_lattice(L):
+    from paper_1401_0188_gb300 import build
+    build.build(debug=True)
+    env = dict(os.environ, LBM13_DEBUG_BUILD="1")
+    r = subprocess.run([sys.executable, "-c", SCRIPT], cwd=ROOT, env=env, capture_output=True, text=True, timeout=1200)
+    assert r.returncode == 0, r.stderr[-3000:]
+    d = json.loads(r.stdout.strip().splitlines()[-1])
+    assert d == {"step": 14, "resident": 14, "barrier": 6, "violations": 0}, d
