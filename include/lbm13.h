@@ -267,8 +267,15 @@ int lbm13_info(lbm13_t h, int64_t out[8]);
  * 288 in FP64) comes from the lattice's allocator at the first such call and is
  * released by lbm13_destroy; where it cannot be allocated, or where
  * lbm13_set_stream has moved a lattice with a caller's allocator to another
- * stream before that call, the lattice steps launch by launch.  Every wait is bounded (1 s); a timeout leaves the
- * state incomplete and is reported as LBM13_ETIMEOUT by the next synchronising
+ * stream before that call, the lattice steps launch by launch.  A launch from
+ * shared memory holds the SMs of its tiles, all of them from about 256^2 nodes on,
+ * for up to 1024 steps (2 to 14 ms): kernels of other streams that find no room
+ * wait for its end.  Many lattices stepped at once on streams of their own share
+ * the GPU better launch by launch (OFF), or as one plan.  Microseconds in which
+ * each of N lattices advances a step, AUTO and OFF, FP32: 64^2 N = 16 5.8 and 7.2;
+ * 128^2 N = 4 3.4 and 3.9, N = 8 6.7 and 4.5; 256^2 N = 2 3.6 and 4.3, N = 4 7.2
+ * and 5.1, N = 16 28.6 and 17.7.
+ * Every wait is bounded (1 s); a timeout leaves the state incomplete and is reported as LBM13_ETIMEOUT by the next synchronising
  * call (lbm13_synchronize, lbm13_residual, lbm13_moments, lbm13_project,
  * lbm13_get_raw_state, lbm13_save).  LBM13_EINVAL for another mode. */
 #define LBM13_PERSISTENT_AUTO 0
@@ -428,7 +435,8 @@ const char *lbm13_plan_last_error(lbm13_plan_t p);
  * whose lattices fit the SMs' shared memory together (about 300,000 nodes in all,
  * no more lattices than SMs) takes n >= 32 steps there, up to 1024 a launch, as
  * lbm13_step does for one lattice (lbm13_set_persistent; results are
- * bit-identical), whatever tile shape is set; not with a lattice that is set to
+ * bit-identical), whatever tile shape is set, and leaves four SMs to kernels of other
+ * streams where that costs at most 5% by its estimate; not with a lattice that is set to
  * LBM13_PERSISTENT_OFF, with LBM13_HALO sides, or on a stream under capture.  The
  * exchange buffers (160 bytes per node) come from the plan's allocator at the first
  * such call; where they cannot be allocated, the plan steps launch by launch.  A

@@ -1758,14 +1758,29 @@ int plan_setup_resident(lbm13_plan_t p)
         bytes += res_exchange_bytes(h->nx, h->ny, 4);
         p->res_states = p->res_states || res_states_pass(h->wf);
     }
+    // on all SMs, and leaving some free for other streams (kResFree)
     std::vector<ResShape> best, shapes;
     double best_t = 0.0;
-    for (int ex : kResPlanWidths) {
-        const double t = res_plan_shapes(lats, 4, p->sms, ex, shapes);
-        if (t > 0.0 && (best_t == 0.0 || t < best_t)) {
-            best_t = t;
-            best = shapes;
-            p->res_ex = ex;
+    const auto split = [&](int sms, std::vector<ResShape> &out, int &width) {
+        double least = 0.0;
+        for (int ex : kResPlanWidths) {
+            const double t = res_plan_shapes(lats, 4, sms, ex, shapes);
+            if (t > 0.0 && (least == 0.0 || t < least)) {
+                least = t;
+                out = shapes;
+                width = ex;
+            }
+        }
+        return least;
+    };
+    best_t = split(p->sms, best, p->res_ex);
+    if (!best.empty() && p->sms > 4 * kResFree) {
+        std::vector<ResShape> less;
+        int width = 0;
+        const double t = split(p->sms - kResFree, less, width);
+        if (t > 0.0 && t <= kResShare * best_t) {
+            best = less;
+            p->res_ex = width;
         }
     }
     if (best.empty()) return LBM13_OK;

@@ -364,6 +364,14 @@ int resident_capacity(const ResShape &s, bool force, const WallArgs<C> *wall);
 // rows of `ex` columns (kResPlanWidths); xchg holds the lattices' exchange buffers
 // at their offsets.  states: evaluate the walls' states once a step
 // (res_states_pass of any of the lattices).
+// A tile may take an SM's registers and shared memory whole, and a launch lasts up to
+// 1024 steps: with a tile on every SM, kernels of other streams wait for its end (a
+// server's admission beside a round of 24 solves, a new 128^2 lattice set and read once,
+// took 3.5 ms instead of 0.45).  A plan leaves kResFree SMs to them where the split that
+// does is at most kResShare times as slow by the estimate: 0.65 ms; the round 5% longer.
+// One lattice does not: a 256^2 cavity would be 9 to 15% slower.
+constexpr int kResFree = 4;
+constexpr double kResShare = 1.05;
 struct ResPlanTile {
     ResShape s;
     int lattice, tile;
