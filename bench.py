@@ -124,6 +124,13 @@ class Clocks:
                 "samples": len(rows), "power_w_max": max(float(r[3]) for r in rows if r[3].replace(".", "").isdigit())}
 
 
+def issue_rate(clocks, sms):
+    """G warp instructions per second that `sms` SMs issue (four a clock each) at the SM
+    clock of a Clocks summary; None without a sample."""
+    mhz = (clocks or {}).get("sm_mhz")
+    return None if not mhz else 4 * sms * mhz * 1e6 / 1e9
+
+
 STEP_SOURCES = ("lbm13_internal.h", "lbm13_math.cuh", "lbm13_fixed.cuh", "lbm13_stepdev.cuh", "lbm13_step.cu")
 PAIR_SOURCES = STEP_SOURCES + ("lbm13_pair.h", "lbm13_mbar.cuh", "lbm13_step2.cu")
 
@@ -503,18 +510,18 @@ def run_ours(args):
         # issue, so its roofline is the issue rate: 4 warp instructions per SM
         # per clock at the SM clock sampled during the timed region
         bytes_lu = 13 * elem
-        clocks = clk.summary() or {}
-        sm_mhz = clocks.get("sm_mhz") or 2070.0
+        clocks = clk.summary()
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
-        issue_peak = 4 * sms * sm_mhz * 1e6 / 1e9
+        issue_peak = issue_rate(clocks, sms)
         ipl = pair_record(f"pair_{args.precision}_warp_instr_per_lu")
         traffic = pair_record(f"pair_{args.precision}_{n}")
         achieved_hbm = bytes_lu * n * n / per_step_s / 1e9
         roofline = {
             "bound": "alu", "unit": "G warp instr/s", "peak": issue_peak, "peak_kind": "derived",
-            "peak_basis": f"4 warp instructions per SM per clock x {sms} SMs x {sm_mhz:.0f} MHz (sampled)",
+            "peak_basis": None if issue_peak is None else
+                f"4 warp instructions per SM per clock x {sms} SMs x {clocks['sm_mhz']:.0f} MHz (sampled)",
             "achieved": None if ipl is None else ipl * n * n / per_step_s / 1e9,
-            "frac": None if ipl is None else ipl * n * n / per_step_s / 1e9 / issue_peak,
+            "frac": None if ipl is None or issue_peak is None else ipl * n * n / per_step_s / 1e9 / issue_peak,
             "instr_per_lu": ipl, "traffic": traffic,
             "hbm": {"achieved": achieved_hbm, "peak": peak, "unit": "GB/s", "frac": achieved_hbm / peak,
                     "bytes_per_lu": bytes_lu, "peak_kind": peak_kind},
@@ -576,7 +583,9 @@ def run_ours(args):
         lat.set_state_device(*f)
         del f
         lat.step(3)
-        ms64 = time_steps(lat, args.fp64_steps, torch)
+        with Clocks(local) as clk_step:  # of this kernel: it draws other power than the FP32 one
+            lat.step(64)  # long enough for a sample (0.2 s)
+            ms64 = time_steps(lat, args.fp64_steps, torch)
         s64 = ms64 / 1e3 / args.fp64_steps
         fp64 = {"value": n * n / s64 / 1e6, "unit": UNIT, "ms_per_step": 1e3 * s64, "steps": args.fp64_steps,
                 "bytes_per_lu": 208, "hbm_gbs": 208 * n * n / s64 / 1e9,
@@ -588,13 +597,13 @@ def run_ours(args):
         ipl = profile_record("step_kernel_fp64_ops.txt", "fp64_warp_instr_per_lu")
         with Clocks(local) as clk64:
             rate, probe_s = lbm13.fp64_fma_rate(1 << 16)
-        sm_mhz = (clk.summary() or {}).get("sm_mhz") or 2070.0
-        issue_peak = 4 * torch.cuda.get_device_properties(local).multi_processor_count * sm_mhz * 1e6 / 1e9
+        issue_peak = issue_rate(clk_step.summary(), torch.cuda.get_device_properties(local).multi_processor_count)
         fp64["roofline"] = {
             "bound": "alu", "unit": "G warp instr/s", "peak": issue_peak, "peak_kind": "derived",
             "achieved": None if ipl is None else ipl * n * n / s64 / 1e9,
-            "frac": None if ipl is None else ipl * n * n / s64 / 1e9 / issue_peak,
+            "frac": None if ipl is None or issue_peak is None else ipl * n * n / s64 / 1e9 / issue_peak,
             "instr_per_lu": ipl,
+            "clocks": clk_step.summary(),
             "fp64_pipe": {
                 "peak": rate / 1e9, "unit": "G FP64 instr/s",
                 "peak_basis": f"lbm13_fp64_fma_rate: 8 independent FMA chains per thread, 8 blocks of 256 per SM, "
