@@ -223,6 +223,17 @@ def test_fp32_readings_are_no_less_exact_than_fp64_arithmetic(lib, params, sizes
     _check_reading(lib, params, sizes, bound, True)
 
 
+@pytest.mark.parametrize("single", [False, True])
+@pytest.mark.parametrize("sizes", [(2e-3, 1e-2, 2e-3), (1e-2, 3e-2, 1e-2), (1e-4, 1e-3, 2e-3), (1e-2, 1e-7, 1e-3), (1e-3, 2e-2, 1e-5)])
+def test_no_reading_leaves_its_range(lib, sizes, single):
+    """A sum beyond 63 bits would be off by a large part of the node's populations: 400,000
+    nodes, the squares of the velocity above the second moment among them."""
+    p = pstar(0.05, 0.71)
+    f = S._states(p, sizes, 400_000, np.random.default_rng(100), 1e-2)
+    v, ei, ep = _read(lib, p, BOUNDS["buoyancy"], f, single)
+    assert (np.abs(ei).max(axis=1) <= 2.0 ** -40 * np.abs(f).max(axis=1)).all()
+
+
 def test_fp32_readings_of_floats_below_the_normal_range(lib):
     """Nodes of 1e-30 and less, some of whose populations are subnormal."""
     p = pstar(0.05, 0.71)
