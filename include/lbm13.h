@@ -274,10 +274,12 @@ int lbm13_info(lbm13_t h, int64_t out[8]);
  * the GPU better launch by launch (OFF), or as one plan.  Microseconds in which
  * each of N lattices advances a step, AUTO and OFF, FP32: 64^2 N = 16 5.8 and 7.2;
  * 128^2 N = 4 3.4 and 3.9, N = 8 6.7 and 4.5; 256^2 N = 2 3.6 and 4.3, N = 4 7.2
- * and 5.1, N = 16 28.6 and 17.7.
- * Every wait is bounded (1 s); a timeout leaves the state incomplete and is reported as LBM13_ETIMEOUT by the next synchronising
- * call (lbm13_synchronize, lbm13_residual, lbm13_moments, lbm13_project,
- * lbm13_get_raw_state, lbm13_save).  LBM13_EINVAL for another mode. */
+ * and 5.1, N = 16 28.6 and 17.7; FP64: 64^2 N = 4 3.8 and 6.1, N = 8 7.8 and 7.0;
+ * 128^2 N = 2 4.2 and 6.2, N = 4 8.2 and 7.7; 256^2 N = 2 12.3 and 9.9, N = 16 98 and
+ * 53.
+ * Every wait is bounded (1 s); a timeout leaves the state incomplete and is reported
+ * as LBM13_ETIMEOUT by the next synchronising call (lbm13_synchronize,
+ * lbm13_residual, lbm13_moments, lbm13_project, lbm13_get_raw_state, lbm13_save).  LBM13_EINVAL for another mode. */
 #define LBM13_PERSISTENT_AUTO 0
 #define LBM13_PERSISTENT_OFF 1
 #define LBM13_PERSISTENT_ON 2

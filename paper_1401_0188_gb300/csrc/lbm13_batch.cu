@@ -32,7 +32,8 @@ namespace {
 // integers, 186 registers if left alone): 24 warps with one row, 16 with two, though
 // words spill; 64 cavities of 128 to 320 squared, one block per tile, microseconds a
 // step without a cap and with 16 / 20 / 24 / 28 warps: one row, BY = 4: 397 and 262 /
-// 249 / 246 / 248, two rows: 406 and 315 / 320 / 331 / 339.
+// 249 / 246 / 248, two rows: 406 and 315 / 320 / 331 / 339.  With the collision as it is
+// now: one row 299 with 24 warps (310 with 20), two rows 411 with 16 (454 with 12).
 constexpr int batch_blocks(int elem, int R, int BY)
 {
     return elem == 4 ? (R == 1 ? 32 / BY : R == 2 ? 24 / BY : 1) : (R == 1 ? 24 / BY : R == 2 ? 16 / BY : 1);

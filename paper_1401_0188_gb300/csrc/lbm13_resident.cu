@@ -12,9 +12,9 @@
 // Microseconds per step, per-step launches (32-step graphs) and this kernel: FP32
 // 64^2 periodic 3.3 and 1.15, 64^2 cavity 4.2 and 1.65, 256^2 cavity 4.9 and 2.3,
 // 1024 x 128 channel 8.0 and 3.4, 512^2 periodic 6.3 and 4.2; FP64 (collision in
-// integers in both) 64^2 periodic 8.5 and 2.6, 256^2 cavity 15.9 and 8.9, 1024 x
-// 128 channel 18.5 and 14.0.  What bounds it is the chain of one node's step (450
-// instructions in FP32, 1150 in FP64, at two to four clocks each with the few
+// integers in both) 64^2 periodic 5.4 and 2.8, 256^2 cavity 10.4 and 9.9, 1024 x
+// 128 channel 14.5 and 15.7.  What bounds it is the chain of one node's step (450
+// instructions in FP32, 1365 in FP64, at two to four clocks each with the few
 // warps that a tile gives) between two barriers; an exchange through flags and
 // fences instead of numbered units took 2.4 us instead of 0.8.
 //
