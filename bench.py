@@ -75,10 +75,14 @@ class Clocks:
          "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
          "clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
 
+    count = 0
+
     def __init__(self, index):
         self.index = index
         self.proc = None
-        self.path = os.path.join(tempfile.gettempdir(), f"lbm13_clocks_{os.getpid()}.csv")
+        # a file of its own: a later region's samples are not this one's
+        Clocks.count += 1
+        self.path = os.path.join(tempfile.gettempdir(), f"lbm13_clocks_{os.getpid()}_{Clocks.count}.csv")
 
     def __enter__(self):
         try:
