@@ -79,13 +79,22 @@ def request_setup(req):
     return req.L, ny, p, W.poiseuille(g, T0=T0, dT=0.01, wall_density=1)
 
 
+# populations that the SMs' shared memory may hold (152 SMs, csrc/lbm13_resident.h)
+SHARED_BYTES = 152 * 222 * 1024
+
+
 def lattice_bytes(nx, ny, precision):
-    """Device bytes a request holds: two population buffers and the FP64
-    reduction buffers (six fields plus per-block partial sums, an upper
-    bound on the library's block count)."""
+    """Device bytes a request holds, an upper bound: two population buffers, the
+    FP64 reduction buffers (six fields plus per-block partial sums, at most the
+    library's block count), for a lattice that may step from shared memory its
+    exchange buffer (two copies of a node's populations in 16-byte units of three
+    words; its share of the plan's, or its own when it steps alone), and small
+    words in allocations of 256 bytes."""
     elem = 8 if precision == lbm13.FP64 else 4
     pitch = (nx + 31) // 32 * 32
-    return 2 * 13 * elem * pitch * ny + 8 * (6 * nx * ny + 1216 * 16 + 32)
+    units = (13 * elem // 4 + 2) // 3
+    exchange = 2 * 16 * units * nx * ny if 13 * elem * nx * ny <= SHARED_BYTES else 0
+    return 2 * 13 * elem * pitch * ny + 8 * (6 * nx * ny + 1216 * 16 + 34) + exchange + 4096
 
 
 def poisson_trace(n, rate, seed=5151, side_range=(64, 192), ra_range=(1e3, 1e5), Pr=0.71, tol=1e-7,

@@ -203,3 +203,14 @@ def test_a_lattice_is_set_up_beside_a_plan_in_shared_memory(L):
         b.close()
     assert min(took) < 2e-3, took
     plan.close()
+
+
+@pytest.mark.parametrize("size", [(64, 64), (187, 211), (256, 256), (360, 360), (700, 600), (901, 803)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_a_lattice_holds_no_more_than_the_server_counts(L, precision, size):
+    from paper_1401_0188_gb300 import serving
+    g = _lattice(L, *size, "cavity", precision, L.PERSISTENT_AUTO)
+    g.step(64)
+    g.residual()
+    assert g.info()["device_bytes"] <= serving.lattice_bytes(*size, precision)
+    g.close()
